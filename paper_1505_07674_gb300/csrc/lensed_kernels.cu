@@ -42,6 +42,7 @@
 #include <utility>
 
 #include "lensed_internal.cuh"
+#include "lensed_pair.cuh"
 #include "lensed_sie_trig.cuh"
 
 namespace lensed {
@@ -457,8 +458,13 @@ __device__ __forceinline__ void sie_row_v(const SieF &k, const RowTerms &R, V x,
     const V v = vfma(dx, vsplat<V>(-k.sn), vfma(dx, vsplat<V>(-k.snl), vsplat<V>(R.dv)));
     const V w = vfma(u, u, vsplat<V>(k.s2));
     const V psi2 = vfma(vsplat<V>(k.q2), w, vfma(vsplat<V>(k.q2l), w, vmul(v, v)));
-    const V psi = vmul(psi2, vmap(psi2, [](float a) { return a > 0.f ? rsqrtf(a) : 0.f; }));
-    const V du = vadd(psi, vsplat<V>(k.s)), dv = vadd(psi, vsplat<V>(k.q2s));
+    // psi + s and psi + q^2 s: a pair forms each with one rounding, a ray
+    // traced alone (the last of a row with an odd number of nodes) rounds psi
+    const V rs = vmap(psi2, [](float a) { return a > 0.f ? rsqrtf(a) : 0.f; });
+    constexpr bool kAlone = std::is_same_v<V, float>;
+    const V psi = vmul(psi2, rs);
+    const V du = kAlone ? vadd(psi, vsplat<V>(k.s)) : vfma(psi2, rs, vsplat<V>(k.s));
+    const V dv = kAlone ? vadd(psi, vsplat<V>(k.q2s)) : vfma(psi2, rs, vsplat<V>(k.q2s));
     V A1, A2;
     if (k.series != 0.f) {
         // q -> 1: atan(e z)/e and atanh(e z)/e by their series in e z
@@ -939,13 +945,6 @@ __device__ __forceinline__ float light_f32_rho(const LightF &k, float x, float y
     return fmaf(k.A, g, k.Al * g);
 }
 
-// MIXED_FF re-traces rays with (R / r)^2 below this.  Measured against the
-// oracle (225 prior points of the 200x200 workload, 256 of the 64x64 one),
-// R < r/2 leaves the largest log-likelihood errors as low as R < r does
-// (7.2e-4 and 4.7e-4 against 9.3e-4 and 3.7e-4: the worst points are set by
-// other float terms) at a quarter of the re-traced rays; below it they grow
-// (R < 0.32 r: 1.1e-3, R < 0.2 r: 3.1e-3 on the 200x200 sample).
-constexpr float kCuspRho2 = 0.25f;
 constexpr int kQCap = 2048;       // deferred float-float rays per trace block
 
 // a2-a5 in FP32 (also the first pass of MIXED): one thread per pixel; for
@@ -1119,10 +1118,78 @@ __device__ __forceinline__ float pixel_rays(const KC &kc, const SysDev &S, int n
     return acc;
 }
 
+// The modes whose first pass keeps no per-ray state (FP32, MIXED, and
+// MIXED_FF with its re-traces in a second pass) trace two pixels per thread
+// (lensed_pair.cuh): their CTAs have half as many threads as the trace block
+// has pixels.  MIXED_FF with in-block re-traces keeps one pixel per thread.
+template <int MODE, bool GQ>
+constexpr bool kTracePairs = MODE != LENSED_PREC_MIXED_FF || GQ;
+
+// trace_item for two pixels per thread: items start + t and start + t +
+// blockDim.x of the block.  Lanes without an item trace the block's last one
+// and write nothing (the warp votes on the form of atanh, so all lanes run).
+template <int G, bool EXACT, bool GQ>
+__device__ __forceinline__ void pair_item(PairSmem &sm, const SysDev *__restrict__ sys,
+                                          const int *__restrict__ comp_type,
+                                          const int *__restrict__ comp_plane,
+                                          const float *__restrict__ cf,
+                                          const unsigned char *__restrict__ valid, int P,
+                                          int C_total, const int *__restrict__ need,
+                                          const NodeTables &nodes, int p0,
+                                          float *__restrict__ Lbuf, long long L_stride,
+                                          const FfQueue &fq, const TraceBlock tb, const int p,
+                                          const bool stage)
+{
+    if (!valid[(size_t)tb.sys * P + p]) return;
+    const SysDev &S = sys[tb.sys];
+    if (stage)
+        stage_pair(sm, S, comp_type, comp_plane, cf, ((size_t)p * C_total + S.comp_off) * kNC,
+                   nodes, EXACT ? kPairW : S.nn);
+    __syncthreads();
+    const int first = tb.start + (int)(threadIdx.x & ~31u);
+    if (first >= tb.end) return;  // a whole warp without items
+    const int ia = tb.start + (int)threadIdx.x, ib = ia + (int)blockDim.x;
+    const bool live_a = ia < tb.end, live_b = ib < tb.end;
+    const int ka = min(ia, tb.end - 1), kb = min(ib, tb.end - 1);
+    const int pa = need ? need[S.need_off + ka] : ka, pb = need ? need[S.need_off + kb] : kb;
+    const int nx = S.nx;
+    const int ra = pa / nx, rb = pb / nx;
+    const float2 jc = make_float2((float)(pa - ra * nx) - S.cx, (float)(pb - rb * nx) - S.cx);
+    const float2 ic = make_float2((float)ra - S.cy, (float)rb - S.cy);
+    float2 acc = sp(0.f);
+    if (nodes.pre_f && S.pre_off >= 0)
+        acc = make_float2(nodes.pre_f[S.pre_off + pa], nodes.pre_f[S.pre_off + pb]);
+    unsigned near = 0u;
+    pair_pixels<G, EXACT, GQ>(sm, S, jc, ic, acc, near);
+    const size_t base = (size_t)(p - p0) * L_stride + S.pix_off;
+    if (live_a) Lbuf[base + pa] = acc.x;
+    if (live_b) Lbuf[base + pb] = acc.y;
+    if (GQ) {
+        // a pixel with a ray inside half an effective radius of a source
+        // centre goes to the pixel queue (one atomic per warp): k_refine_ff
+        // recomputes it with those rays deferred.  Every other pixel's sum is
+        // final here.
+        const unsigned full = 0xffffffffu, lane = threadIdx.x & 31u;
+        const bool fa = live_a && (near & 1u), fb = live_b && (near & 2u);
+        const unsigned ba = __ballot_sync(full, fa), bb = __ballot_sync(full, fb);
+        if (ba | bb) {
+            unsigned long long e = 0ull;
+            if (lane == 0u) e = atomicAdd(fq.cnt + 1, (unsigned long long)(__popc(ba) + __popc(bb)));
+            e = __shfl_sync(full, e, 0);
+            const unsigned below = (1u << lane) - 1u;
+            const unsigned long long ea = e + __popc(ba & below), eb = e + __popc(ba) + __popc(bb & below);
+            if (fa && ea < (unsigned long long)fq.pcap)
+                fq.pix[ea] = FfEntry{(unsigned)(base + pa), (unsigned)tb.sys};
+            if (fb && eb < (unsigned long long)fq.pcap)
+                fq.pix[eb] = FfEntry{(unsigned)(base + pb), (unsigned)tb.sys};
+        }
+    }
+}
+
 // The work of one trace block tb at point p (every thread of the CTA calls
 // it; it returns to the caller, which may take another item).  stage = false:
 // the shared constants already hold tb's system at point p.
-template <int MODE, int G, bool EXACT, bool GQ>
+template <int MODE, int G, bool EXACT>
 __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
                                            const int *__restrict__ comp_type,
                                            const int *__restrict__ comp_plane,
@@ -1132,7 +1199,7 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
                                            int C_total, const int *__restrict__ need,
                                            const NodeTables &nodes, int p0,
                                            float *__restrict__ Lbuf, long long L_stride,
-                                           const FfQueue &fq, const TraceBlock tb, const int p,
+                                           const TraceBlock tb, const int p,
                                            const bool stage = true)
 {
     __shared__ __align__(16) TraceSmem sm;
@@ -1140,12 +1207,9 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
     const SysDev &S = sys[tb.sys];
     const size_t cbase = ((size_t)p * C_total + S.comp_off) * kNC;
     // MIXED_FF with at most 8 nodes per row defers its float-float re-traces
-    // (64-bit ray mask per pixel): to a block-wide queue processed by all
-    // lanes after the main loop, or (GQ) to the launch's global queue; the
-    // others re-trace in place
-    constexpr bool kFfDefer = (MODE == LENSED_PREC_MIXED_FF) && EXACT;
-    constexpr bool kQueue = kFfDefer && !GQ;
-    constexpr bool kWarpQ = kFfDefer && GQ;
+    // (64-bit ray mask per pixel) to a block-wide queue processed by all
+    // lanes after the main loop; with more it re-traces in place
+    constexpr bool kQueue = (MODE == LENSED_PREC_MIXED_FF) && EXACT;
     __shared__ int q_n;
     __shared__ unsigned short q_t[kQueue ? kQCap : 1];
     __shared__ unsigned char q_r[kQueue ? kQCap : 1];
@@ -1156,8 +1220,7 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
 
     const int idx = tb.start + threadIdx.x;
     const bool active = idx < tb.end;
-    // (a warp appending to the global queue needs all its lanes)
-    if (!kQueue && !kWarpQ && !active) return;
+    if (!kQueue && !active) return;
     const int ncomp = S.ncomp;
     const int nn = EXACT ? G : S.nn;
     const int nx = S.nx;
@@ -1170,32 +1233,10 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
     float pmin = kCuspRho2;          // smallest (R/r)^2 of the pixel's rays
     constexpr int kNear = MODE != LENSED_PREC_MIXED_FF ? kNearIgnore
                         : !EXACT                     ? kNearInPlace
-                        : GQ                         ? kNearFlag
                                                      : kNearDefer;
     if (active)
         acc = pixel_rays<MODE, G, EXACT, kNear>(SmemConsts{sm}, S, ncomp, nn, jc, ic, acc, mask,
                                                 pmin);
-    if (kWarpQ) {
-        // a pixel with a ray inside half an effective radius of a source
-        // centre goes to the pixel queue (one atomic per warp): k_refine_ff
-        // recomputes it with those rays deferred.  Every other pixel's sum is
-        // final here (the same arithmetic as the deferring loop, which leaves
-        // a pixel without such rays unchanged).
-        const unsigned full = 0xffffffffu, lane = threadIdx.x & 31u;
-        const bool flag = active && pmin < kCuspRho2;
-        const unsigned ball = __ballot_sync(full, flag);
-        const size_t lin = (size_t)(p - p0) * L_stride + S.pix_off + pix;
-        if (ball) {
-            unsigned long long base = 0ull;
-            if (lane == 0u) base = atomicAdd(fq.cnt + 1, (unsigned long long)__popc(ball));
-            base = __shfl_sync(full, base, 0);
-            const unsigned long long e = base + (unsigned long long)__popc(ball & ((1u << lane) - 1u));
-            if (flag && e < (unsigned long long)fq.pcap)
-                fq.pix[e] = FfEntry{(unsigned)lin, (unsigned)tb.sys};
-        }
-        if (active) Lbuf[lin] = acc;
-        return;
-    }
     if (kQueue) {
         // each pixel's deferred rays take consecutive slots in ray order
         const int n_t = __popcll(mask);
@@ -1236,7 +1277,7 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
 }
 
 template <int MODE, int G, bool EXACT, bool GQ>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs<MODE, GQ> ? 6 : 0)
     k_trace_rows(const SysDev *__restrict__ sys, const int *__restrict__ comp_type,
                  const int *__restrict__ comp_plane, const float *__restrict__ cf,
                  const double *__restrict__ cd, const unsigned char *__restrict__ valid, int P,
@@ -1244,9 +1285,16 @@ __global__ void __launch_bounds__(256)
                  NodeTables nodes, int p0, float *__restrict__ Lbuf, long long L_stride,
                  FfQueue fq)
 {
-    trace_item<MODE, G, EXACT, GQ>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total, need,
-                                   nodes, p0, Lbuf, L_stride, fq, blocks[blockIdx.x],
+    if constexpr (kTracePairs<MODE, GQ>) {
+        __shared__ __align__(16) PairSmem sm;
+        pair_item<G, EXACT, GQ>(sm, sys, comp_type, comp_plane, cf, valid, P, C_total, need, nodes,
+                                p0, Lbuf, L_stride, fq, blocks[blockIdx.x], p0 + (int)blockIdx.y,
+                                true);
+    } else {
+        trace_item<MODE, G, EXACT>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total, need,
+                                   nodes, p0, Lbuf, L_stride, blocks[blockIdx.x],
                                    p0 + (int)blockIdx.y);
+    }
 }
 
 // The same work as a persistent, work-queued launch: a grid sized to the
@@ -1256,33 +1304,36 @@ __global__ void __launch_bounds__(256)
 // point changes.
 constexpr int kPqGrab = 4;
 template <int MODE, int G, bool EXACT, bool GQ>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs<MODE, GQ> ? 6 : 0)
     k_trace_rows_pq(const SysDev *__restrict__ sys, const int *__restrict__ comp_type,
                     const int *__restrict__ comp_plane, const float *__restrict__ cf,
                     const double *__restrict__ cd, const unsigned char *__restrict__ valid, int P,
                     int C_total, const TraceBlock *__restrict__ blocks,
                     const int *__restrict__ need, NodeTables nodes, int p0,
                     float *__restrict__ Lbuf, long long L_stride, FfQueue fq, int n_blocks,
-                    long long n_items, unsigned long long *__restrict__ work)
+                    unsigned n_items, unsigned long long *__restrict__ work)
 {
-    __shared__ long long s_item;
-    int cur_sys = -1, cur_p = -1;
+    __shared__ unsigned s_item;
+    __shared__ __align__(16) std::conditional_t<kTracePairs<MODE, GQ>, PairSmem, char> sm;
     for (;;) {
-        if (threadIdx.x == 0) s_item = (long long)atomicAdd(work, (unsigned long long)kPqGrab);
+        if (threadIdx.x == 0) s_item = (unsigned)atomicAdd(work, (unsigned long long)kPqGrab);
         __syncthreads();
-        const long long first = s_item;
+        const unsigned first = s_item;
         __syncthreads();  // read by all before thread 0 takes the next ones
         if (first >= n_items) return;
-        const long long last = min(first + kPqGrab, n_items);
-        for (long long item = first; item < last; ++item) {
-            const int q = (int)(item / n_blocks);
-            const TraceBlock tb = blocks[item - (long long)q * n_blocks];
-            const int p = p0 + q;
-            trace_item<MODE, G, EXACT, GQ>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total,
-                                           need, nodes, p0, Lbuf, L_stride, fq, tb, p,
-                                           tb.sys != cur_sys || p != cur_p);
-            cur_sys = tb.sys;
-            cur_p = p;
+        const unsigned last = min(first + (unsigned)kPqGrab, n_items);
+#pragma unroll 1
+        for (unsigned item = first; item < last; ++item) {
+            const unsigned q = item / (unsigned)n_blocks;
+            const TraceBlock tb = blocks[item - q * (unsigned)n_blocks];
+            // (a system's blocks follow one another from pixel 0 on)
+            const bool stage = item % (unsigned)kPqGrab == 0u || tb.start == 0;
+            if constexpr (kTracePairs<MODE, GQ>)
+                pair_item<G, EXACT, GQ>(sm, sys, comp_type, comp_plane, cf, valid, P, C_total, need,
+                                        nodes, p0, Lbuf, L_stride, fq, tb, p0 + (int)q, stage);
+            else
+                trace_item<MODE, G, EXACT>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total,
+                                           need, nodes, p0, Lbuf, L_stride, tb, p0 + (int)q, stage);
             __syncthreads();  // the item is done with the shared arrays
         }
     }
@@ -1466,7 +1517,10 @@ static void trace_rows_t(int threads, const SysDev *sys, const int *comp_type,
                          void *Lbuf, long long L_stride, cudaStream_t st, FfQueue fq,
                          unsigned long long *work)
 {
-    if (!work) {
+    if (kTracePairs<MODE, GQ>) threads /= 2;
+    const long long n_items = (long long)n_blocks * nP;
+    // (the work-queued form counts its items in 32 bits)
+    if (!work || n_items > (1LL << 31)) {
         dim3 grid((unsigned)n_blocks, (unsigned)nP);
         k_trace_rows<MODE, G, EXACT, GQ><<<grid, threads, 0, st>>>(
             sys, comp_type, comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0,
@@ -1476,13 +1530,12 @@ static void trace_rows_t(int threads, const SysDev *sys, const int *comp_type,
     int per_sm = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace_rows_pq<MODE, G, EXACT, GQ>,
                                                   threads, 0);
-    const long long n_items = (long long)n_blocks * nP;
     const long long want = (long long)std::max(g_sm_count, 1) * std::max(per_sm, 1);
     const unsigned grid = (unsigned)std::max(1LL, std::min(want, n_items));
     cudaMemsetAsync(work, 0, sizeof(unsigned long long), st);
     k_trace_rows_pq<MODE, G, EXACT, GQ><<<grid, threads, 0, st>>>(
         sys, comp_type, comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0,
-        (float *)Lbuf, L_stride, fq, n_blocks, n_items, work);
+        (float *)Lbuf, L_stride, fq, n_blocks, (unsigned)n_items, work);
 }
 
 // GQ: the launch has a global float-float queue (MIXED_FF, at most 8 nodes per row)
