@@ -89,7 +89,7 @@ struct TraceBlock {
 // on the parameter point (see kPlanePrecomputed), at SysDev::pre_off; NULL
 // while that table is being computed.
 struct NodeTables {
-    const float *u, *w;
+    const float *u, *ul, *w;  // ul: the residual of u (ud ~ u + ul)
     const double *ud, *wd;
     const float *pre_f;
     const double *pre_d;
@@ -120,8 +120,8 @@ struct LaunchCfg {
 
 // One deferred float-float ray of a trace launch: lin = the pixel's index in
 // the launch's image scratch ((point - p0) * stride + pixel offset of the
-// system + pixel), sr = system << 8 | ray index in the rule grid (row-major,
-// b * nn + a).  A pixel's entries are consecutive and in ray order.
+// system + pixel), sr = system << 6 | b << 3 | a, (a, b) the ray's nodes along x
+// and y (at most 8 nodes per row).  A pixel's entries are consecutive and in ray order.
 // lin == kFfNone marks a slot left empty.
 struct FfEntry {
     unsigned lin, sr;

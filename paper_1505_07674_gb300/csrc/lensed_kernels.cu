@@ -843,13 +843,6 @@ struct FfConsts {
     const int *type, *plane;
 };
 
-// A node offset (FP64) as a float pair.
-__device__ __forceinline__ ff node_pair(double v)
-{
-    const float hi = (float)v;
-    return {hi, (float)(v - (double)hi)};
-}
-
 // Source-plane brightness of a ray of pixel (jc, ic) with node offsets ua
 // (along x) and vb (along y) as float pairs, with the lens equation in
 // float-float (all lens components) and the light in FP32.  Every constant
@@ -977,8 +970,7 @@ struct SmemConsts {
 struct GlobalConsts {
     const float *cfp;
     const int *typ, *pln;
-    const float *uu, *ww;
-    const double *ud;
+    const float *uu, *ul, *ww;
     __device__ const float *cf(int c) const { return cfp + c * kNC; }
     __device__ int plane(int c) const { return pln[c]; }
     __device__ int type(int c) const { return typ[c]; }
@@ -987,7 +979,7 @@ struct GlobalConsts {
     __device__ float ff(int ncomp, float jc, float ic, float h, float h_lo, int a, int b) const
     {
         return source_brightness_ff_at(FfConsts{cfp, typ, pln}, ncomp, jc, ic, h, h_lo,
-                                       node_pair(ud[a]), node_pair(ud[b]));
+                                       lensed::ff{uu[a], ul[a]}, lensed::ff{uu[b], ul[b]});
     }
 };
 
@@ -1378,7 +1370,8 @@ __global__ void __launch_bounds__(kFfThreads)
         const float jc = (float)j - S.cx, ic = (float)i - S.cy;
         const GlobalConsts K{cf + ((size_t)p * C_total + S.comp_off) * kNC,
                              comp_type + S.comp_off, comp_plane + S.comp_off,
-                             nodes.u + S.node_off, nodes.w + S.w2_off, nodes.ud + S.node_off};
+                             nodes.u + S.node_off, nodes.ul + S.node_off,
+                             nodes.w + S.w2_off};
         unsigned long long mask = 0ull;
         float acc = 0.f, pmin = kCuspRho2;
         if (active) {
@@ -1402,9 +1395,10 @@ __global__ void __launch_bounds__(kFfThreads)
             unsigned long long q = base + (unsigned long long)(incl - n_t);
             if (base + (unsigned long long)total <= cap) {
                 if (active) fq.prun[e] = make_uint2((unsigned)q, (unsigned)n_t);
-                const unsigned sys8 = s << 8;
-                for (unsigned long long m = mask; m; m &= m - 1ull, ++q)
-                    fq.ent[q] = FfEntry{lin, sys8 | (unsigned)(__ffsll((long long)m) - 1)};
+                for (unsigned long long m = mask; m; m &= m - 1ull, ++q) {
+                    const unsigned r = (unsigned)(__ffsll((long long)m) - 1);
+                    fq.ent[q] = FfEntry{lin, s << 6 | r / G << 3 | r % G};
+                }
             } else {
                 if (active) fq.prun[e] = make_uint2(0u, 0u);
                 for (int k = 0; k < n_t; ++k, ++q)
@@ -1441,17 +1435,16 @@ __global__ void __launch_bounds__(kFfThreads)
          e += (long long)gridDim.x * blockDim.x) {
         const FfEntry E = fq.ent[e];
         if (E.lin == kFfNone) continue;
-        const SysDev &S = sys[E.sr >> 8];
-        const int r = (int)(E.sr & 255u), nn = S.nn;
+        const SysDev &S = sys[E.sr >> 6];
+        const int a = (int)(E.sr & 7u), b = (int)(E.sr >> 3 & 7u);
         const unsigned q = E.lin / L_stride;
-        const int pix = (int)(E.lin - q * L_stride) - S.pix_off;
+        const int pix = (int)(E.lin - q * L_stride) - (int)S.pix_off;
         const int i = pix / S.nx, j = pix - i * S.nx;
-        const int a = r % nn, b = r / nn;
         const FfConsts K{cf + ((size_t)(p0 + (int)q) * C_total + S.comp_off) * kNC,
                          comp_type + S.comp_off, comp_plane + S.comp_off};
+        const float *u = nodes.u + S.node_off, *ul = nodes.ul + S.node_off;
         fq.val[e] = source_brightness_ff_at(K, S.ncomp, (float)j - S.cx, (float)i - S.cy, S.h,
-                                            S.h_lo, node_pair(nodes.ud[S.node_off + a]),
-                                            node_pair(nodes.ud[S.node_off + b]));
+                                            S.h_lo, ff{u[a], ul[a]}, ff{u[b], ul[b]});
     }
 }
 
@@ -1467,10 +1460,13 @@ __global__ void k_apply_ff(const SysDev *__restrict__ sys, NodeTables nodes,
         const uint2 run = fq.prun[e];
         if (run.y == 0u) continue;
         const FfEntry R = fq.pix[e];
-        const int w2 = sys[R.sr].w2_off;
+        const SysDev &S = sys[R.sr];
+        const float *w = nodes.w + S.w2_off;
         float acc = Lbuf[R.lin];
-        for (unsigned k = 0; k < run.y; ++k)
-            acc = fmaf(nodes.w[w2 + (int)(fq.ent[run.x + k].sr & 255u)], fq.val[run.x + k], acc);
+        for (unsigned k = 0; k < run.y; ++k) {
+            const unsigned sr = fq.ent[run.x + k].sr;
+            acc = fmaf(w[(sr >> 3 & 7u) * (unsigned)S.nn + (sr & 7u)], fq.val[run.x + k], acc);
+        }
         Lbuf[R.lin] = acc;
     }
 }
