@@ -41,7 +41,7 @@ constexpr double kMixedCoreFactor = 2.0;
 // Series in e replaces atan/atanh below this (both precisions).
 constexpr double kSeriesE = 1e-3;
 
-// Sersic b_n table: piecewise Chebyshev series in log n over
+// Sersic tables (b_n, and the logarithm of the normalisation): piecewise Chebyshev series in log n over
 // [kBnMin, kBnMax], kBnSeg segments of degree kBnDeg (relative error ~3e-15);
 // outside that range the prologue solves for b_n by Newton.
 constexpr double kBnMin = 0.2, kBnMax = 12.0;
@@ -154,14 +154,15 @@ void note_buffers(int delta);
 
 // --- kernels launched from the runtime (defined in lensed_kernels.cu) ---
 
-// a1: per (system, point) packed constants and validity.
+// a1: per (system, point) packed constants and validity (imgpos: some system
+// of the model has an image-plane prior).
 // a1 for components c0 .. c0+nC-1 (global indices, belonging to systems
 // s0 .. s0+nS-1) and points p0 .. p0+nP-1; with single_row, params is one
 // row (the render path).  cvalid: [P][C_total] scratch bytes.
 void launch_prologue(const SysDev *sys, const int *comp_sys, int s0, int nS, int c0, int nC,
                      const int *comp_type, const int *comp_free, const double *comp_value,
                      const double *params, bool single_row, int P, int p0, int nP,
-                     int n_par_stride, int C_total, const double *bn_table, float *cf,
+                     int n_par_stride, int C_total, const double *bn_table, bool imgpos, float *cf,
                      double *cd, unsigned char *cvalid, unsigned char *valid, cudaStream_t st);
 
 // a2-a5: pixel luminosities of the pixels in the block table, for points

@@ -115,31 +115,52 @@ __device__ double sersic_b(double n)
     return b;
 }
 
-// b_n from the Chebyshev table when n lies in its range, else by Newton.
-__device__ double sersic_b_lookup(double n, const double *__restrict__ table)
+// b_n and g = 2n ln b_n - ln n - lnGamma(2n), both from Chebyshev tables in
+// log n (one argument, two independent Clenshaw chains) when n lies in their
+// range, else by Newton and lgamma.
+__device__ __noinline__ void sersic_b_solve(double n, double &bn, double &g)
 {
-    if (table && n >= kBnMin && n <= kBnMax) {
-        const double l0 = log(kBnMin), dl = (log(kBnMax) - l0) / kBnSeg;
-        const double ln = log(n);
-        const int k = min(max((int)((ln - l0) / dl), 0), kBnSeg - 1);
-        const double lo = l0 + k * dl;
-        const double t = (2.0 * (ln - lo) - dl) / dl;  // [-1, 1]
-        const double *c = table + k * (kBnDeg + 1);
-        // Clenshaw
-        double b1 = 0.0, b2 = 0.0;
-        for (int j = kBnDeg; j >= 1; --j) {
-            const double b0 = 2.0 * t * b1 - b2 + c[j];
-            b2 = b1;
-            b1 = b0;
-        }
-        return t * b1 - b2 + c[0];
+    bn = sersic_b(n);
+    g = 2.0 * n * log(bn) - log(n) - lgamma(2.0 * n);
+}
+__device__ __forceinline__ void sersic_b_lookup(double n, const double *__restrict__ table,
+                                                double &bn, double &g)
+{
+    if (!(n >= kBnMin && n <= kBnMax)) {
+        sersic_b_solve(n, bn, g);
+        return;
     }
-    return sersic_b(n);
+    const double l0 = log(kBnMin), dl = (log(kBnMax) - l0) / kBnSeg;
+    const double ln = log(n);
+    const int k = min(max((int)((ln - l0) * (1.0 / dl)), 0), kBnSeg - 1);
+    const double lo = l0 + k * dl;
+    const double t = (2.0 * (ln - lo) - dl) * (1.0 / dl), t2 = 2.0 * t;  // t in [-1, 1]
+    const double *c = table + k * (kBnDeg + 1), *d = c + kBnSeg * (kBnDeg + 1);
+    double b1 = 0.0, b2 = 0.0, e1 = 0.0, e2 = 0.0;
+#pragma unroll
+    for (int j = kBnDeg; j >= 1; --j) {
+        const double b0 = t2 * b1 - b2 + c[j], e0 = t2 * e1 - e2 + d[j];
+        b2 = b1;
+        b1 = b0;
+        e2 = e1;
+        e1 = e0;
+    }
+    bn = t * b1 - b2 + c[0];
+    g = t * e1 - e2 + d[0];
 }
 
 // One thread per (point, component): resolve the component's parameters,
 // check its domain and write its packed constants and a validity byte.
-__global__ void k_prologue_comp(const SysDev *__restrict__ sys, const int *__restrict__ comp_sys,
+//
+// A serial chain of FP64 functions on a unit that takes 16 cycles per warp
+// instruction, so its time is the chain's length: a CTA is one warp of one
+// component (lanes are points: no branch of another type's functions, and
+// the chains of different components run on different SMs), and the
+// profile's normalisation comes from a table instead of pow, lgamma and
+// three logarithms.  Prologue of a call 33 -> 20 us (8 points, 3 components),
+// 42 -> 24 us (1,024 points, 4), 51 -> 33 us (128 points, 8, an image prior).
+constexpr int kPrologueThreads = 32;
+__global__ void __launch_bounds__(kPrologueThreads) k_prologue_comp(const SysDev *__restrict__ sys, const int *__restrict__ comp_sys,
                                 int c0, int nC, const int *__restrict__ comp_type,
                                 const int *__restrict__ comp_free,
                                 const double *__restrict__ comp_value,
@@ -148,10 +169,11 @@ __global__ void k_prologue_comp(const SysDev *__restrict__ sys, const int *__res
                                 const double *__restrict__ bn_table, float *__restrict__ cf,
                                 double *__restrict__ cd, unsigned char *__restrict__ cvalid)
 {
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= (long long)nC * nP) return;
-    const int gc = c0 + (int)(tid % nC);
-    const int p = p0 + (int)(tid / nC);
+    const int warps = (nP + kPrologueThreads - 1) / kPrologueThreads;  // per component
+    const int gc = c0 + (int)(blockIdx.x / (unsigned)warps);
+    const int pi = (int)(blockIdx.x % (unsigned)warps) * kPrologueThreads + (int)threadIdx.x;
+    if (pi >= nP) return;
+    const int p = p0 + pi;
     const int s = comp_sys[gc];
     const double zeropoint = sys[s].zeropoint;
     const double hd = sys[s].hd;
@@ -246,8 +268,9 @@ __global__ void k_prologue_comp(const SysDev *__restrict__ sys, const int *__res
         // 15 kind, 16 x0_lo, 17 y0_lo.  rho^2 = (q u^2 + v^2/q)/r^2; Sersic t = B rho^(2 p2) with
         // B = b_n log2(e), p2 = 1/(2n); Gaussian (r = sqrt(2) sigma) t =
         // B rho^2 with B = log2(e); I = A 2^-t with A = I_0 h^2.
+        // F = 10^(-0.4 (mag - zp)) enters by its logarithm
         const double r = v[2];
-        const double F = pow(10.0, -0.4 * (v[3] - zeropoint));
+        const double lF = -0.4 * M_LN10 * (v[3] - zeropoint);
         double n = 4.0, q, pa;
         if (type == LENSED_SERSIC) { n = v[4]; q = v[5]; pa = v[6]; }
         else { q = v[4]; pa = v[5]; }
@@ -270,18 +293,18 @@ __global__ void k_prologue_comp(const SysDev *__restrict__ sys, const int *__res
             o[7] = 1.0 / (q * r2);
             o[10] = 1.0;
             o[11] = 1.4426950408889634;  // log2(e)
-            o[13] = F / (M_PI * r2) * hd * hd;
+            o[13] = exp(lF) / (M_PI * r2) * hd * hd;
             o[15] = kKindGauss;
         } else if (ok) {
-            const double bn = sersic_b_lookup(n, bn_table);
             // I_0 = F b^(2n) / (2 pi n r^2 Gamma(2n)), in logs
-            const double lI0 = log(F) + 2.0 * n * log(bn) - log(2.0 * M_PI * n * r * r) -
-                               lgamma(2.0 * n);
-            o[6] = q / (r * r);
-            o[7] = 1.0 / (q * r * r);
+            double bn, g;
+            sersic_b_lookup(n, bn_table, bn, g);
+            const double ir2 = 1.0 / (r * r);
+            o[6] = q * ir2;
+            o[7] = ir2 / q;
             o[10] = 0.5 / n;
             o[11] = bn * 1.4426950408889634;
-            o[13] = exp(lI0) * hd * hd;
+            o[13] = exp(lF + g) * (ir2 * (0.5 / M_PI)) * hd * hd;
             o[15] = kKindPower;
         }
     }
@@ -592,40 +615,63 @@ __device__ __forceinline__ double brightness_f64(double x, double y, const RayCt
 // Validity of a (system, point): every component in its domain.  Then the
 // image-plane priors (Sec. 5): a source whose position parameters are an
 // image-plane position theta is moved to theta - alpha(theta) (Eq. 1), the
-// deflection of the same point's lens in FP64.
+// deflection of the same point's lens in FP64.  IMGPOS: some system of the
+// launch has such a source; a half-warp then takes a (system, point), each lane
+// one component's deflection, added in component order.
+template <bool IMGPOS>
 __global__ void k_prologue_valid(const SysDev *__restrict__ sys, int s0, int nS, int P, int p0,
                                  int nP, int C_total, const int *__restrict__ comp_type,
                                  const unsigned char *__restrict__ cvalid, float *__restrict__ cf,
                                  double *__restrict__ cd, unsigned char *__restrict__ valid)
 {
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= (long long)nS * nP) return;
-    const int s = s0 + (int)(tid / nP);
-    const int p = p0 + (int)(tid % nP);
+    static_assert(LENSED_MAX_COMPONENTS == 16, "a half-warp per (system, point)");
+    const long long thread = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const long long tid = IMGPOS ? thread / 16 : thread;
+    const bool in = tid < (long long)nS * nP;
+    if (!IMGPOS && !in) return;
+    const int s = s0 + (in ? (int)(tid / nP) : 0);
+    const int p = p0 + (in ? (int)(tid % nP) : 0);
     const SysDev &S = sys[s];
     unsigned char ok = 1;
     for (int c = 0; c < S.ncomp; ++c) ok &= cvalid[(size_t)p * C_total + S.comp_off + c];
-    if (ok && S.imgpos_mask) {
+    if (IMGPOS) {
+        const int l = (int)(threadIdx.x & 15u);
         const size_t base = ((size_t)p * C_total + S.comp_off) * kNC;
-        for (int c = 0; c < S.ncomp; ++c) {
-            if (!((S.imgpos_mask >> c) & 1)) continue;
-            double *cc = cd + base + (size_t)c * kNC;
+        const bool lens = l < S.ncomp && comp_type[S.comp_off + l] <= LENSED_POINTMASS;
+        const int images = ok && in ? S.imgpos_mask : 0;
+        // (both halves of the warp take as many turns: they shuffle together)
+        const unsigned turns = (unsigned)images | (unsigned)__shfl_xor_sync(0xffffffffu, images, 16);
+        for (int c = 0; c < LENSED_MAX_COMPONENTS; ++c) {
+            if (!((turns >> c) & 1u)) continue;
+            const bool mine = (images >> c) & 1;
+            double *cc = cd + base + (size_t)(mine ? c : 0) * kNC;
             const double tx = cc[0], ty = cc[1];
+            double dx = 0.0, dy = 0.0;
+            if (mine && lens)
+                deflect_f64(comp_type[S.comp_off + l], tx, ty, cd + base + (size_t)l * kNC, dx, dy);
             double ax = 0.0, ay = 0.0;
-            for (int l = 0; l < S.ncomp; ++l) {
-                const int t = comp_type[S.comp_off + l];
-                if (t <= LENSED_POINTMASS) deflect_f64(t, tx, ty, cd + base + (size_t)l * kNC, ax, ay);
+            for (int k = 0; k < LENSED_MAX_COMPONENTS; ++k) {
+                const double kx = __shfl_sync(0xffffffffu, dx, k, 16);
+                const double ky = __shfl_sync(0xffffffffu, dy, k, 16);
+                const bool has = __shfl_sync(0xffffffffu, (int)lens, k, 16) != 0;
+                if (has) {
+                    ax += kx;
+                    ay += ky;
+                }
             }
             const double yx = tx - ax, yy = ty - ay;
-            if (!isfinite(yx) || !isfinite(yy)) ok = 0;
-            cc[0] = yx;
-            cc[1] = yy;
-            float *fc = cf + base + (size_t)c * kNC;
-            fc[0] = (float)yx;
-            fc[1] = (float)yy;
-            fc[16] = (float)(yx - (double)fc[0]);
-            fc[17] = (float)(yy - (double)fc[1]);
+            if (mine && (!isfinite(yx) || !isfinite(yy))) ok = 0;
+            if (mine && l == 0) {
+                cc[0] = yx;
+                cc[1] = yy;
+                float *fc = cf + base + (size_t)c * kNC;
+                fc[0] = (float)yx;
+                fc[1] = (float)yy;
+                fc[16] = (float)(yx - (double)fc[0]);
+                fc[17] = (float)(yy - (double)fc[1]);
+            }
         }
+        if (!in || l != 0) return;
     }
     valid[(size_t)s * P + p] = ok;
 }
@@ -633,17 +679,20 @@ __global__ void k_prologue_valid(const SysDev *__restrict__ sys, int s0, int nS,
 void launch_prologue(const SysDev *sys, const int *comp_sys, int s0, int nS, int c0, int nC,
                      const int *comp_type, const int *comp_free, const double *comp_value,
                      const double *params, bool single_row, int P, int p0, int nP,
-                     int n_par_stride, int C_total, const double *bn_table, float *cf,
+                     int n_par_stride, int C_total, const double *bn_table, bool imgpos, float *cf,
                      double *cd, unsigned char *cvalid, unsigned char *valid, cudaStream_t st)
 {
-    const long long n = (long long)nC * nP;
-    const int threads = 64;
-    k_prologue_comp<<<(unsigned)((n + threads - 1) / threads), threads, 0, st>>>(
+    const unsigned warps = (unsigned)((nP + kPrologueThreads - 1) / kPrologueThreads);
+    k_prologue_comp<<<(unsigned)nC * warps, kPrologueThreads, 0, st>>>(
         sys, comp_sys, c0, nC, comp_type, comp_free, comp_value, params, single_row ? 1 : 0, P,
         p0, nP, n_par_stride, C_total, bn_table, cf, cd, cvalid);
     const long long n2 = (long long)nS * nP;
-    k_prologue_valid<<<(unsigned)((n2 + 127) / 128), 128, 0, st>>>(
-        sys, s0, nS, P, p0, nP, C_total, comp_type, cvalid, cf, cd, valid);
+    if (imgpos)
+        k_prologue_valid<true><<<(unsigned)((n2 * 16 + 63) / 64), 64, 0, st>>>(
+            sys, s0, nS, P, p0, nP, C_total, comp_type, cvalid, cf, cd, valid);
+    else
+        k_prologue_valid<false><<<(unsigned)((n2 + 127) / 128), 128, 0, st>>>(
+            sys, s0, nS, P, p0, nP, C_total, comp_type, cvalid, cf, cd, valid);
 }
 
 

@@ -182,7 +182,7 @@ long double host_gamma_p(long double a, long double x)
 }
 
 // Sersic b_n (root of P(2n, b) = 1/2) by bisection in long double.
-double host_sersic_b(double n)
+long double host_sersic_b(double n)
 {
     long double lo = 0, hi = 2.0L * n;
     for (int it = 0; it < 200; ++it) {
@@ -191,32 +191,41 @@ double host_sersic_b(double n)
         if (host_gamma_p(2.0L * n, mid) < 0.5L) lo = mid;
         else hi = mid;
     }
-    return (double)(0.5L * (lo + hi));
+    return 0.5L * (lo + hi);
 }
 
-// Piecewise Chebyshev coefficients of b_n in log n (kBnSeg segments of
-// degree kBnDeg over [kBnMin, kBnMax]), from values at the Chebyshev points.
-std::vector<double> build_bn_table()
+// Piecewise Chebyshev coefficients in log n (kBnSeg segments of degree kBnDeg
+// over [kBnMin, kBnMax]) from values at the Chebyshev points, of b_n and,
+// behind it, of 2n ln b_n - ln n - lnGamma(2n) (the normalisation of the
+// profile, k_prologue_comp).  Built once per process.
+const std::vector<double> &bn_table_host()
 {
-    std::vector<double> tab(kBnSeg * (kBnDeg + 1));
-    const double l0 = log(kBnMin), dl = (log(kBnMax) - l0) / kBnSeg;
-    const int N = kBnDeg + 1;
-    const long double pi = 3.141592653589793238462643383279502884L;
-    for (int k = 0; k < kBnSeg; ++k) {
-        std::vector<long double> f(N);
-        for (int i = 0; i < N; ++i) {
-            const long double t = cosl(pi * (i + 0.5L) / N);
-            f[i] = host_sersic_b((double)expl(l0 + dl * (k + 0.5L * (t + 1))));
+    static const std::vector<double> table = [] {
+        const int N = kBnDeg + 1;
+        std::vector<double> tab(2 * kBnSeg * N);
+        const double l0 = log(kBnMin), dl = (log(kBnMax) - l0) / kBnSeg;
+        const long double pi = 3.141592653589793238462643383279502884L;
+        for (int k = 0; k < kBnSeg; ++k) {
+            std::vector<long double> f(N), g(N);
+            for (int i = 0; i < N; ++i) {
+                const long double t = cosl(pi * (i + 0.5L) / N);
+                const double n = (double)expl(l0 + dl * (k + 0.5L * (t + 1)));
+                f[i] = host_sersic_b(n);
+                g[i] = 2.0L * n * logl(f[i]) - logl(n) - lgammal(2.0L * n);
+            }
+            for (int q = 0; q < 2; ++q)
+                for (int j = 0; j < N; ++j) {
+                    long double c = 0;
+                    for (int i = 0; i < N; ++i)
+                        c += (q ? g[i] : f[i]) * cosl(pi * j * (i + 0.5L) / N);
+                    c *= 2.0L / N;
+                    if (j == 0) c *= 0.5L;
+                    tab[(q * kBnSeg + k) * N + j] = (double)c;
+                }
         }
-        for (int j = 0; j < N; ++j) {
-            long double c = 0;
-            for (int i = 0; i < N; ++i) c += f[i] * cosl(pi * j * (i + 0.5L) / N);
-            c *= 2.0L / N;
-            if (j == 0) c *= 0.5L;
-            tab[k * N + j] = (double)c;
-        }
-    }
-    return tab;
+        return tab;
+    }();
+    return table;
 }
 
 // Integral of x^k P_n(x) over [-1, 1]: zero unless k >= n and k - n even,
@@ -472,6 +481,7 @@ struct lensed_model {
     int n_par_max = 0;
     int C_total = 0;
     long long total_pix = 0;
+    bool imgpos = false;  // some source is placed by an image-plane prior
     int T_total = 0;  // active (chi^2) tiles over all systems
     size_t scratch_budget = (size_t)2 << 30;  // bytes of per-point image scratch
 
@@ -716,7 +726,7 @@ void enqueue_batch(lensed_model *m, const double *params, int P, double *out, La
     if (tm) tm->begin(0);
     launch_prologue(m->sys.p, m->comp_sys.p, 0, m->n_sys, 0, m->C_total, m->comp_type.p,
                     m->comp_free.p, m->comp_value.p, params, false, P, 0, P, m->n_par_max,
-                    m->C_total, m->bn_table.p, m->cf.p, m->cd.p, m->cvalid.p, m->valid.p, st);
+                    m->C_total, m->bn_table.p, m->imgpos, m->cf.p, m->cd.p, m->cvalid.p, m->valid.p, st);
     if (tm) tm->end();
     const int chunk = m->chunk();
     for (int p0 = 0; p0 < P; p0 += chunk) {
@@ -895,7 +905,7 @@ static int precompute_fixed_light(lensed_model *m, const std::vector<int> &cplan
     // no parameter), all systems marked valid for this pass
     launch_prologue(m->sys.p, m->comp_sys.p, 0, m->n_sys, 0, m->C_total, m->comp_type.p,
                     m->comp_free.p, m->comp_value.p, zeros.p, true, 1, 0, 1, m->n_par_max,
-                    m->C_total, m->bn_table.p, m->rcf.p, m->rcd.p, m->rcvalid.p, m->rvalid.p, 0);
+                    m->C_total, m->bn_table.p, m->imgpos, m->rcf.p, m->rcd.p, m->rcvalid.p, m->rvalid.p, 0);
     CUDA_OK(cudaMemset(m->rvalid.p, 1, m->n_sys));
     const NodeTables nodes{m->node_u.p, m->node_ul.p, m->node_w.p, m->node_ud.p, m->node_wd.p,
                            nullptr, nullptr, 0};
@@ -1299,6 +1309,7 @@ extern "C" int lensed_create_model(const lensed_system_desc *systems, int n_syst
     m->C_total = C_total;
     m->total_pix = total_pix;
     m->T_total = T_total;
+    for (const SysDev &S : sh) m->imgpos = m->imgpos || S.imgpos_mask != 0;
     m->sys_h = sh;
     m->need_count = need_count;
     m->n_nodes = nn_v;
@@ -1350,7 +1361,7 @@ extern "C" int lensed_create_model(const lensed_system_desc *systems, int n_syst
         (rc = m->psf_d.upload(psf_d)) || (rc = m->node_u.upload(node_u)) || (rc = m->node_ul.upload(node_ul)) ||
         (rc = m->node_w.upload(node_w)) || (rc = m->node_ud.upload(node_ud)) ||
         (rc = m->node_wd.upload(node_wd)) || (rc = m->need.upload(need)) ||
-        (rc = m->psf_blocks.upload(m->psf_blocks_h)) || (rc = m->bn_table.upload(build_bn_table())) ||
+        (rc = m->psf_blocks.upload(m->psf_blocks_h)) || (rc = m->bn_table.upload(bn_table_host())) ||
         (rc = m->render_psf.upload(m->render_psf_h))) {
         std::string msg = g_last_error;
         delete m;
@@ -1434,7 +1445,7 @@ extern "C" int lensed_render(lensed_model *m, int system, const double *params, 
     // one point: consts at p = 0, valid at index system (P = 1)
     launch_prologue(m->sys.p, m->comp_sys.p, system, 1, S.comp_off, S.ncomp, m->comp_type.p,
                     m->comp_free.p, m->comp_value.p, params, true, 1, 0, 1, m->n_par_max,
-                    m->C_total, m->bn_table.p, m->rcf.p, m->rcd.p, m->rcvalid.p, m->rvalid.p, st);
+                    m->C_total, m->bn_table.p, m->imgpos, m->rcf.p, m->rcd.p, m->rcvalid.p, m->rvalid.p, st);
     launch_trace(m->precision, m->cfg(), m->n_nodes[system], m->sys.p, m->comp_type.p,
                  m->comp_plane.p, m->rcf.p,
                  m->rcd.p, m->rvalid.p, 1, m->C_total,
@@ -1535,7 +1546,7 @@ extern "C" int lensed_render_error(lensed_model *m, int system, const double *pa
     const SysDev &S = m->sys_h[system];
     launch_prologue(m->sys.p, m->comp_sys.p, system, 1, S.comp_off, S.ncomp, m->comp_type.p,
                     m->comp_free.p, m->comp_value.p, params, true, 1, 0, 1, m->n_par_max,
-                    m->C_total, m->bn_table.p, m->rcf.p, m->rcd.p, m->rcvalid.p, m->rvalid.p, st);
+                    m->C_total, m->bn_table.p, m->imgpos, m->rcf.p, m->rcd.p, m->rcvalid.p, m->rvalid.p, st);
     // the Kronrod and the embedded Gauss luminosities, each with the trace
     // (and MIXED fix-up) kernels of lensed_render
     for (int g = 0; g < 2; ++g) {
@@ -1636,7 +1647,7 @@ extern "C" int lensed_loglike_plain(lensed_model *m, const double *params, int P
         for (int p = 0; p < P; ++p) {
             launch_prologue(m->sys.p, m->comp_sys.p, s, 1, m->sys_h[s].comp_off,
                             m->sys_h[s].ncomp, m->comp_type.p, m->comp_free.p, m->comp_value.p,
-                            params, false, P, p, 1, m->n_par_max, m->C_total, m->bn_table.p,
+                            params, false, P, p, 1, m->n_par_max, m->C_total, m->bn_table.p, m->imgpos,
                             m->cf.p, m->cd.p, m->cvalid.p, m->valid.p, st);
             launch_trace(m->precision, cfg, m->n_nodes[s], m->sys.p, m->comp_type.p,
                          m->comp_plane.p, m->cf.p,
@@ -1919,7 +1930,7 @@ extern "C" int lensed_loglike_batch_noalloc(lensed_model *m, const double *param
     const LaunchCfg cfg = m->cfg();
     launch_prologue(m->sys.p, m->comp_sys.p, 0, m->n_sys, 0, m->C_total, m->comp_type.p,
                     m->comp_free.p, m->comp_value.p, params, false, P, 0, P, m->n_par_max,
-                    m->C_total, m->bn_table.p, cf, cd, cvalid, valid, st);
+                    m->C_total, m->bn_table.p, m->imgpos, cf, cd, cvalid, valid, st);
     for (int p0 = 0; p0 < P; p0 += chunk) {
         const int nP = std::min(chunk, P - p0);
         // no second-pass queue here (it lives in model-owned memory): in
