@@ -1964,6 +1964,43 @@ static __host__ __device__ __forceinline__ int psf_row_stride(int q)
     return (kTileW + 2 * q + 3) & ~3;
 }
 
+// The direct kernel's staged tile: rows of an odd number of 16-byte quads, so
+// that the eight rows one phase of its 16-byte reads touches (16 lanes on 16
+// rows, same columns) fall on different banks.  With two lanes per row on an
+// even number of quads every read was a two-way conflict, and the kernel was
+// bound by shared memory instead of the FMA pipe: PSF stage 250 -> 207 us
+// (400x400, 15x15 taps, 100 points), 425 -> 416 us (200x200, 21x21 taps, 1,024
+// points), 305 -> 297 us (161x143, 21x21, 700 points).
+template <typename T>
+static __host__ __device__ __forceinline__ int psf_conv_stride(int q)
+{
+    return psf_row_stride(q) | (int)(16 / sizeof(T));
+}
+
+// N values by 16-byte reads (src 16-byte aligned, N * sizeof(T) a multiple of 16)
+template <int N>
+__device__ __forceinline__ void read_quads(float *dst, const float *src)
+{
+#pragma unroll
+    for (int k = 0; k < N / 4; ++k) {
+        const float4 v = reinterpret_cast<const float4 *>(src)[k];
+        dst[4 * k] = v.x;
+        dst[4 * k + 1] = v.y;
+        dst[4 * k + 2] = v.z;
+        dst[4 * k + 3] = v.w;
+    }
+}
+template <int N>
+__device__ __forceinline__ void read_quads(double *dst, const double *src)
+{
+#pragma unroll
+    for (int k = 0; k < N / 2; ++k) {
+        const double2 v = reinterpret_cast<const double2 *>(src)[k];
+        dst[2 * k] = v.x;
+        dst[2 * k + 1] = v.y;
+    }
+}
+
 // The separable kernel's strides.  Staged tile: psf_row_stride with an odd
 // number of 16-byte quads, so the two rows one 8-lane phase of its row pass
 // reads fall on different banks.  Row-pass output: 72 floats, 18 quads (2
@@ -2032,7 +2069,7 @@ __global__ void __launch_bounds__(kPsfThreads)
     const bool ok = valid[(size_t)pb.sys * P + p] != 0;
     const int Ph = S.psf_p;
     const int rows = kTileH + 2 * Ph;
-    const int stride = psf_row_stride(Q);
+    const int stride = psf_conv_stride<T>(Q);
     T *s_F = s_L + (size_t)rows * stride;
     const int nx = S.nx, ny = S.ny;
 
@@ -2058,10 +2095,10 @@ __global__ void __launch_bounds__(kPsfThreads)
     __syncthreads();
 
     // each warp owns a 16 x 16 block of outputs (the tile is 2 x 4 warps);
-    // each lane 8 consecutive outputs of one row
+    // each lane 8 consecutive outputs of one row, 16 lanes to the 16 rows
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int tr = (warp >> 2) * 16 + (lane >> 1);
-    const int tcol = (warp & 3) * 16 + (lane & 1) * kOutPerThread;
+    const int tr = (warp >> 2) * 16 + (lane & 15);
+    const int tcol = (warp & 3) * 16 + (lane >> 4) * kOutPerThread;
     const int i = pb.i0 + tr;
     const int jb = pb.j0 + tcol;
     // chi^2 mode: a warp none of whose outputs carries weight skips the
@@ -2071,13 +2108,11 @@ __global__ void __launch_bounds__(kPsfThreads)
 #pragma unroll
     for (int o = 0; o < kOutPerThread; ++o) acc[o] = T(0);
     for (int kk = 0; live && kk <= 2 * Ph; ++kk) {
-        T f[WS];
-#pragma unroll
-        for (int l = 0; l < WS; ++l) f[l] = s_F[kk * WS + l];
-        const T *srow = s_L + (tr + kk) * stride + tcol;
-        T lv[kOutPerThread + 2 * Q];
-#pragma unroll
-        for (int m = 0; m < kOutPerThread + 2 * Q; ++m) lv[m] = srow[m];
+        // (a row segment of up to two values more, inside the staged row)
+        constexpr int LV = (kOutPerThread + 2 * Q + 3) & ~3;
+        T f[WS], lv[LV];
+        read_quads<WS>(f, s_F + kk * WS);
+        read_quads<LV>(lv, s_L + (tr + kk) * stride + tcol);
         // each PSF row is summed on its own and then added to the output: the
         // float rounding of the sum grows like sqrt(rows) + sqrt(taps per
         // row) instead of sqrt(all taps), which on a 21 x 21 PSF cuts its
@@ -2289,7 +2324,7 @@ static constexpr int kPsfSepSmemMax =
 
 // Largest dynamic shared memory a k_psf instance can ask for (Q = P = 15, FP64).
 static constexpr int kPsfSmemMax =
-    ((kTileH + 2 * LENSED_MAX_PSF_HALF) * ((kTileW + 2 * LENSED_MAX_PSF_HALF + 3) & ~3) +
+    ((kTileH + 2 * LENSED_MAX_PSF_HALF) * ((kTileW + 2 * LENSED_MAX_PSF_HALF + 3) & ~3 | 2) +
      (2 * LENSED_MAX_PSF_HALF + 1) * ((2 * LENSED_MAX_PSF_HALF + 1 + 3) & ~3)) *
     (int)sizeof(double);
 
@@ -2380,7 +2415,7 @@ static void psf_launch_t(int p_max, const SysDev *sys, const T *psf, const T *da
                          long long L_stride, double *partial, int T_total, float *out,
                          cudaStream_t st)
 {
-    const size_t smem = ((size_t)(kTileH + 2 * p_max) * psf_row_stride(Q) +
+    const size_t smem = ((size_t)(kTileH + 2 * p_max) * psf_conv_stride<T>(Q) +
                          (size_t)(2 * p_max + 1) * psf_tap_stride(Q)) * sizeof(T);
     dim3 grid((unsigned)n_blocks, (unsigned)nP);
     k_psf<T, Q><<<grid, kPsfThreads, smem, st>>>(sys, psf, data, weight, valid, P, blocks, p0,
