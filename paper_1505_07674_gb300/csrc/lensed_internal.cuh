@@ -156,6 +156,8 @@ void note_buffers(int delta);
 
 // a1: per (system, point) packed constants and validity (imgpos: some system
 // of the model has an image-plane prior).
+// zero2 / zero1 (if not NULL): counters zeroed on the way, two and one (the
+// second pass's and the work queue's of the trace launch that follows).
 // a1 for components c0 .. c0+nC-1 (global indices, belonging to systems
 // s0 .. s0+nS-1) and points p0 .. p0+nP-1; with single_row, params is one
 // row (the render path).  cvalid: [P][C_total] scratch bytes.
@@ -163,19 +165,21 @@ void launch_prologue(const SysDev *sys, const int *comp_sys, int s0, int nS, int
                      const int *comp_type, const int *comp_free, const double *comp_value,
                      const double *params, bool single_row, int P, int p0, int nP,
                      int n_par_stride, int C_total, const double *bn_table, bool imgpos, float *cf,
-                     double *cd, unsigned char *cvalid, unsigned char *valid, cudaStream_t st);
+                     double *cd, unsigned char *cvalid, unsigned char *valid, cudaStream_t st,
+                     unsigned long long *zero2 = nullptr, unsigned long long *zero1 = nullptr);
 
 // a2-a5: pixel luminosities of the pixels in the block table, for points
 // p0 .. p0 + nP - 1, into Lbuf[(p - p0) * L_stride + pix_off + pix].  Every
 // system in the table has nn nodes per row of its rule.  MIXED_FF with
 // cfg.ff_split and a queue (q.cnt != nullptr): the float-float re-traces run
-// in a second kernel after the first (same results bit for bit).
+// in a second kernel after the first (same results bit for bit).  zeroed: the
+// prologue has zeroed the counters of q and work.
 void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const int *comp_type,
                   const int *comp_plane, const float *cf, const double *cd,
                   const unsigned char *valid, int P, int C_total, const TraceBlock *blocks,
                   int n_blocks, const int *need, NodeTables nodes, int p0, int nP, void *Lbuf,
                   long long L_stride, cudaStream_t st, FfQueue q = FfQueue{},
-                  unsigned long long *work = nullptr);
+                  unsigned long long *work = nullptr, bool zeroed = false);
 
 // One-time kernel attributes (dynamic shared memory limits); call before
 // any launch or capture.
@@ -183,7 +187,8 @@ void init_kernel_attributes();
 
 // MIXED only: recompute, with the FP64 SIE, the pixels of each (system,
 // point) that the MIXED rule assigns to FP64 (after launch_trace wrote
-// their FP32 values).  need == nullptr: every pixel of the systems (render).
+// their FP32 values; it follows a trace launch on st, beside which it starts).
+// need == nullptr: every pixel of the systems (render).
 void launch_fix64(LaunchCfg cfg, const SysDev *sys, int s0, int nS, const int *comp_type,
                   const int *comp_plane, const float *cf, const double *cd,
                   const unsigned char *valid, int P, int C_total, const int *need,

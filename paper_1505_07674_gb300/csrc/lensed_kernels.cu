@@ -48,6 +48,44 @@
 namespace lensed {
 
 // ---------------------------------------------------------------------------
+// launches
+
+// Programmatic dependent launch: a kernel launched by `chain` may start while
+// the kernel before it in the stream still runs (once all of that one's
+// blocks have started and called chain_next, or exited), so its launch and
+// prologue cost no gap.  Every block calls chain_wait before it touches
+// anything that an earlier kernel of the stream reads or writes: that returns
+// when the earlier kernel has completed, which by the same rule has waited for
+// the one before it.  Eight points of a 64 x 64 image, a call: 87 us launch by
+// launch, 69 us so; a render with its error map: 283 and 212 us.  The kernels
+// of a second pass are launched without it: their grids are sized to the whole
+// chip, and started as a trace drains, the first idle multiprocessors would
+// take most of their blocks (1,024 points of a 200 x 200 image, trace stage:
+// 1.65 ms so, 1.68 ms chained).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next()
+{
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... K, class... A>
+static void chain(void (*kernel)(K...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                  A &&...args)
+{
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
+// ---------------------------------------------------------------------------
 // math helpers
 
 // MUFU base-2 exponential and logarithm (PTX ex2.approx / lg2.approx, flush
@@ -169,6 +207,8 @@ __global__ void __launch_bounds__(kPrologueThreads) k_prologue_comp(const SysDev
                                 const double *__restrict__ bn_table, float *__restrict__ cf,
                                 double *__restrict__ cd, unsigned char *__restrict__ cvalid)
 {
+    chain_wait();
+    chain_next();
     const int warps = (nP + kPrologueThreads - 1) / kPrologueThreads;  // per component
     const int gc = c0 + (int)(blockIdx.x / (unsigned)warps);
     const int pi = (int)(blockIdx.x % (unsigned)warps) * kPrologueThreads + (int)threadIdx.x;
@@ -622,8 +662,17 @@ template <bool IMGPOS>
 __global__ void k_prologue_valid(const SysDev *__restrict__ sys, int s0, int nS, int P, int p0,
                                  int nP, int C_total, const int *__restrict__ comp_type,
                                  const unsigned char *__restrict__ cvalid, float *__restrict__ cf,
-                                 double *__restrict__ cd, unsigned char *__restrict__ valid)
+                                 double *__restrict__ cd, unsigned char *__restrict__ valid,
+                                 unsigned long long *__restrict__ zero2,
+                                 unsigned long long *__restrict__ zero1)
 {
+    chain_wait();
+    chain_next();
+    // the counters of the call's first trace launch
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (zero2) zero2[0] = zero2[1] = 0ull;
+        if (zero1) *zero1 = 0ull;
+    }
     static_assert(LENSED_MAX_COMPONENTS == 16, "a half-warp per (system, point)");
     const long long thread = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long tid = IMGPOS ? thread / 16 : thread;
@@ -680,19 +729,20 @@ void launch_prologue(const SysDev *sys, const int *comp_sys, int s0, int nS, int
                      const int *comp_type, const int *comp_free, const double *comp_value,
                      const double *params, bool single_row, int P, int p0, int nP,
                      int n_par_stride, int C_total, const double *bn_table, bool imgpos, float *cf,
-                     double *cd, unsigned char *cvalid, unsigned char *valid, cudaStream_t st)
+                     double *cd, unsigned char *cvalid, unsigned char *valid, cudaStream_t st,
+                     unsigned long long *zero2, unsigned long long *zero1)
 {
     const unsigned warps = (unsigned)((nP + kPrologueThreads - 1) / kPrologueThreads);
-    k_prologue_comp<<<(unsigned)nC * warps, kPrologueThreads, 0, st>>>(
-        sys, comp_sys, c0, nC, comp_type, comp_free, comp_value, params, single_row ? 1 : 0, P,
-        p0, nP, n_par_stride, C_total, bn_table, cf, cd, cvalid);
+    chain(k_prologue_comp, (unsigned)nC * warps, kPrologueThreads, 0, st, sys, comp_sys, c0, nC,
+          comp_type, comp_free, comp_value, params, single_row ? 1 : 0, P, p0, nP, n_par_stride,
+          C_total, bn_table, cf, cd, cvalid);
     const long long n2 = (long long)nS * nP;
     if (imgpos)
-        k_prologue_valid<true><<<(unsigned)((n2 * 16 + 63) / 64), 64, 0, st>>>(
-            sys, s0, nS, P, p0, nP, C_total, comp_type, cvalid, cf, cd, valid);
+        chain(k_prologue_valid<true>, (unsigned)((n2 * 16 + 63) / 64), 64, 0, st, sys, s0, nS,
+              P, p0, nP, C_total, comp_type, cvalid, cf, cd, valid, zero2, zero1);
     else
-        k_prologue_valid<false><<<(unsigned)((n2 + 127) / 128), 128, 0, st>>>(
-            sys, s0, nS, P, p0, nP, C_total, comp_type, cvalid, cf, cd, valid);
+        chain(k_prologue_valid<false>, (unsigned)((n2 + 127) / 128), 128, 0, st, sys, s0, nS, P,
+              p0, nP, C_total, comp_type, cvalid, cf, cd, valid, zero2, zero1);
 }
 
 
@@ -1326,6 +1376,8 @@ __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs
                  NodeTables nodes, int p0, float *__restrict__ Lbuf, long long L_stride,
                  FfQueue fq)
 {
+    chain_wait();
+    chain_next();
     if constexpr (kTracePairs<MODE, GQ>) {
         __shared__ __align__(16) PairSmem sm;
         pair_item<G, EXACT, GQ>(sm, sys, comp_type, comp_plane, cf, valid, P, C_total, need, nodes,
@@ -1354,6 +1406,8 @@ __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs
                     float *__restrict__ Lbuf, long long L_stride, FfQueue fq, int n_blocks,
                     unsigned n_items, unsigned long long *__restrict__ work)
 {
+    chain_wait();
+    chain_next();
     __shared__ unsigned s_item;
     __shared__ __align__(16) std::conditional_t<kTracePairs<MODE, GQ>, PairSmem, char> sm;
     for (;;) {
@@ -1567,9 +1621,9 @@ static void trace_rows_t(int threads, const SysDev *sys, const int *comp_type,
     // (the work-queued form counts its items in 32 bits)
     if (!work || n_items > (1LL << 31)) {
         dim3 grid((unsigned)n_blocks, (unsigned)nP);
-        k_trace_rows<MODE, G, EXACT, GQ><<<grid, threads, 0, st>>>(
-            sys, comp_type, comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0,
-            (float *)Lbuf, L_stride, fq);
+        chain(k_trace_rows<MODE, G, EXACT, GQ>, grid, threads, 0, st, sys, comp_type,
+              comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0, (float *)Lbuf,
+              L_stride, fq);
         return;
     }
     int per_sm = 0;
@@ -1577,10 +1631,9 @@ static void trace_rows_t(int threads, const SysDev *sys, const int *comp_type,
                                                   threads, 0);
     const long long want = (long long)std::max(g_sm_count, 1) * std::max(per_sm, 1);
     const unsigned grid = (unsigned)std::max(1LL, std::min(want, n_items));
-    cudaMemsetAsync(work, 0, sizeof(unsigned long long), st);
-    k_trace_rows_pq<MODE, G, EXACT, GQ><<<grid, threads, 0, st>>>(
-        sys, comp_type, comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0,
-        (float *)Lbuf, L_stride, fq, n_blocks, (unsigned)n_items, work);
+    chain(k_trace_rows_pq<MODE, G, EXACT, GQ>, grid, threads, 0, st, sys, comp_type, comp_plane,
+          cf, cd, valid, P, C_total, blocks, need, nodes, p0, (float *)Lbuf, L_stride, fq,
+          n_blocks, (unsigned)n_items, work);
 }
 
 // GQ: the launch has a global float-float queue (MIXED_FF, at most 8 nodes per row)
@@ -1614,10 +1667,12 @@ void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const
                   const int *comp_plane, const float *cf, const double *cd,
                   const unsigned char *valid, int P, int C_total, const TraceBlock *blocks,
                   int n_blocks, const int *need, NodeTables nodes, int p0, int nP, void *Lbuf,
-                  long long L_stride, cudaStream_t st, FfQueue q, unsigned long long *work)
+                  long long L_stride, cudaStream_t st, FfQueue q, unsigned long long *work,
+                  bool zeroed)
 {
     if (n_blocks <= 0 || nP <= 0) return;
     if (!cfg.persistent) work = nullptr;
+    if (work && !zeroed) cudaMemsetAsync(work, 0, sizeof(unsigned long long), st);
     if (precision == LENSED_PREC_FP64) {
         dim3 grid((unsigned)n_blocks, (unsigned)nP);
         k_trace_f64<<<grid, cfg.trace_threads, 0, st>>>(sys, comp_type, comp_plane, cf, cd,
@@ -1630,7 +1685,7 @@ void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const
                            nn <= 8 &&
                            (long long)nP * L_stride < (long long)kFfNone;
         if (split) {
-            cudaMemsetAsync(q.cnt, 0, 2 * sizeof(unsigned long long), st);
+            if (!zeroed) cudaMemsetAsync(q.cnt, 0, 2 * sizeof(unsigned long long), st);
             trace_rows_dispatch<LENSED_PREC_MIXED_FF, true>(
                 nn, cfg.trace_threads, sys, comp_type, comp_plane, cf, cd, valid, P, C_total,
                 blocks, n_blocks, need, nodes, p0, nP, Lbuf, L_stride, st, q, work);
@@ -1801,6 +1856,7 @@ __device__ void fix_pixels(const TraceSmem &sm, const SysDev &S, const int *s_pi
             s_ray[t] = ray_mixed(sm, S, i, j, r % nn, r / nn, ff);
         }
         __syncthreads();
+        chain_wait();
         for (int k = threadIdx.x; k < m; k += blockDim.x) {
             float acc = pre ? pre[s_pix[b0 + k]] : 0.f;
             for (int r = 0; r < nr; ++r) acc = fmaf(sm.w[r], s_ray[k * nr + r], acc);
@@ -1817,6 +1873,10 @@ __global__ void __launch_bounds__(128)
                   int C_total, const int *__restrict__ need, NodeTables nodes, int p0,
                   float *__restrict__ Lbuf, long long L_stride)
 {
+    // the constants are there (the trace kernel waited for the prologue before
+    // it let this one start), so the rays are computed beside the trace; only
+    // writing pixels has to wait for it
+    chain_next();
     __shared__ __align__(16) TraceSmem sm;
     __shared__ float s_ray[kFixRays];
     __shared__ int s_pix[kFixRays];
@@ -1825,7 +1885,10 @@ __global__ void __launch_bounds__(128)
     const int slice = blockIdx.z, slices = gridDim.z;
     const int s = s0 + blockIdx.x;
     const int p = p0 + blockIdx.y;
-    if (!valid[(size_t)s * P + p]) return;
+    if (!valid[(size_t)s * P + p]) {
+        chain_wait();
+        return;
+    }
     const SysDev &S = sys[s];
     const size_t cbase = ((size_t)p * C_total + S.comp_off) * kNC;
     stage_point(sm, S, comp_type, comp_plane, cf, cd, cbase, true, false, nodes);
@@ -1847,6 +1910,7 @@ __global__ void __launch_bounds__(128)
             __syncthreads();
             fix_pixels(sm, S, s_pix, m, s_ray, s_list, s_m, L, pre, nodes.ff != 0);
         }
+        chain_wait();
         return;
     }
     // core discs, one SIE after the other; a pixel already covered by an
@@ -1883,6 +1947,7 @@ __global__ void __launch_bounds__(128)
             fix_pixels(sm, S, s_pix, n, s_ray, s_list, s_m, L, pre, nodes.ff != 0);
         }
     }
+    chain_wait();
 }
 
 void launch_fix64(LaunchCfg cfg, const SysDev *sys, int s0, int nS, const int *comp_type,
@@ -1896,8 +1961,8 @@ void launch_fix64(LaunchCfg cfg, const SysDev *sys, int s0, int nS, const int *c
     const long long pairs = (long long)nS * nP;
     const unsigned slices = pairs * 2 > std::max(1, g_sm_count) ? 1u : (unsigned)kFixSlices;
     dim3 grid((unsigned)nS, (unsigned)nP, slices);
-    k_trace_fix64<<<grid, 128, 0, st>>>(sys, s0, comp_type, comp_plane, cf, cd, valid, P, C_total,
-                                         need, nodes, p0, (float *)Lbuf, L_stride);
+    chain(k_trace_fix64, grid, 128, 0, st, sys, s0, comp_type, comp_plane, cf, cd, valid, P,
+          C_total, need, nodes, p0, (float *)Lbuf, L_stride);
 }
 
 // ---------------------------------------------------------------------------
@@ -2060,6 +2125,8 @@ __global__ void __launch_bounds__(kPsfThreads)
           int p0, const T *__restrict__ Lbuf, long long L_stride, double *__restrict__ partial,
           int T_total, float *__restrict__ out)
 {
+    chain_wait();
+    chain_next();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *s_L = reinterpret_cast<T *>(smem_raw);
     constexpr int W = 2 * Q + 1;
@@ -2185,6 +2252,8 @@ __global__ void __launch_bounds__(kPsfThreads, 4)
               int p0, const float *__restrict__ Lbuf, long long L_stride,
               double *__restrict__ partial, int T_total, float *__restrict__ out)
 {
+    chain_wait();
+    chain_next();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     constexpr int W = 2 * Q + 1;
     constexpr int WS = (W + 3) & ~3;
@@ -2433,8 +2502,8 @@ static void psf_sep_launch_t(int p_max, int r_max, const SysDev *sys, const floa
                          (size_t)r_max * (2 * p_max + 1) + (size_t)r_max * psf_tap_stride(Q)) *
                         sizeof(float);
     dim3 grid((unsigned)n_blocks, (unsigned)nP);
-    k_psf_sep<Q><<<grid, kPsfThreads, smem, st>>>(sys, psf, data, weight, valid, P, blocks, p0,
-                                                   Lbuf, L_stride, partial, T_total, out);
+    chain(k_psf_sep<Q>, grid, kPsfThreads, smem, st, sys, psf, data, weight, valid, P, blocks,
+          p0, Lbuf, L_stride, partial, T_total, out);
 }
 
 template <int... Qs>
@@ -2461,8 +2530,8 @@ static void psf_launch_t(int p_max, const SysDev *sys, const T *psf, const T *da
     const size_t smem = ((size_t)(kTileH + 2 * p_max) * psf_conv_stride<T>(Q) +
                          (size_t)(2 * p_max + 1) * psf_tap_stride(Q)) * sizeof(T);
     dim3 grid((unsigned)n_blocks, (unsigned)nP);
-    k_psf<T, Q><<<grid, kPsfThreads, smem, st>>>(sys, psf, data, weight, valid, P, blocks, p0,
-                                                  Lbuf, L_stride, partial, T_total, out);
+    chain(k_psf<T, Q>, grid, kPsfThreads, smem, st, sys, psf, data, weight, valid, P, blocks,
+          p0, Lbuf, L_stride, partial, T_total, out);
 }
 
 template <typename T>
@@ -2526,6 +2595,8 @@ __global__ void k_finalize(const SysDev *__restrict__ sys, const unsigned char *
                            int P, const double *__restrict__ partial, int T_total,
                            double *__restrict__ out, int s0, int p0, int nS, int nP)
 {
+    chain_wait();
+    chain_next();
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (tid >= (long long)nS * nP) return;
     const int s = s0 + (int)(tid / nP);
@@ -2549,13 +2620,15 @@ void launch_finalize(const SysDev *sys, const unsigned char *valid, int P,
 {
     const long long n = (long long)nS * nP;
     const int threads = 128;
-    k_finalize<<<(unsigned)((n + threads - 1) / threads), threads, 0, st>>>(
-        sys, valid, P, partial, T_total, out, s0, p0, nS, nP);
+    chain(k_finalize, (unsigned)((n + threads - 1) / threads), threads, 0, st, sys, valid, P,
+          partial, T_total, out, s0, p0, nS, nP);
 }
 
 __global__ void k_copy_image(int fp64, const void *__restrict__ Lbuf, long long off, int npix,
                              const unsigned char *__restrict__ valid, float *__restrict__ out)
 {
+    chain_wait();
+    chain_next();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= npix) return;
     if (!valid[0]) {
@@ -2568,14 +2641,16 @@ __global__ void k_copy_image(int fp64, const void *__restrict__ Lbuf, long long 
 void launch_copy_image(int precision, const void *Lbuf, long long off, int npix,
                        const unsigned char *valid, float *out, cudaStream_t st)
 {
-    k_copy_image<<<(npix + 255) / 256, 256, 0, st>>>(precision == LENSED_PREC_FP64, Lbuf, off,
-                                                      npix, valid, out);
+    chain(k_copy_image, (npix + 255) / 256, 256, 0, st, precision == LENSED_PREC_FP64, Lbuf,
+          off, npix, valid, out);
 }
 
 __global__ void k_error_image(int fp64, const void *__restrict__ LK, const void *__restrict__ LG,
                               long long off, int npix, const unsigned char *__restrict__ valid,
                               float *__restrict__ out)
 {
+    chain_wait();
+    chain_next();
     const int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= npix) return;
     if (!valid[0]) {
@@ -2589,8 +2664,8 @@ __global__ void k_error_image(int fp64, const void *__restrict__ LK, const void 
 void launch_error_image(int precision, const void *LK, const void *LG, long long off, int npix,
                         const unsigned char *valid, float *out, cudaStream_t st)
 {
-    k_error_image<<<(npix + 255) / 256, 256, 0, st>>>(precision == LENSED_PREC_FP64, LK, LG, off,
-                                                       npix, valid, out);
+    chain(k_error_image, (npix + 255) / 256, 256, 0, st, precision == LENSED_PREC_FP64, LK, LG,
+          off, npix, valid, out);
 }
 
 }  // namespace lensed

@@ -726,20 +726,24 @@ void enqueue_batch(lensed_model *m, const double *params, int P, double *out, La
     if (tm) tm->begin(0);
     launch_prologue(m->sys.p, m->comp_sys.p, 0, m->n_sys, 0, m->C_total, m->comp_type.p,
                     m->comp_free.p, m->comp_value.p, params, false, P, 0, P, m->n_par_max,
-                    m->C_total, m->bn_table.p, m->imgpos, m->cf.p, m->cd.p, m->cvalid.p, m->valid.p, st);
+                    m->C_total, m->bn_table.p, m->imgpos, m->cf.p, m->cd.p, m->cvalid.p, m->valid.p, st,
+                    m->ffq_cnt.p, m->work.p);
     if (tm) tm->end();
+    bool zeroed = true;  // the counters of the first trace launch
     const int chunk = m->chunk();
     for (int p0 = 0; p0 < P; p0 += chunk) {
         const int nP = std::min(chunk, P - p0);
         if (tm) tm->begin(1);
         // (a second pass, where launch_trace runs one, completes before the
         // MIXED fix-up overwrites its pixels: both are on stream st)
-        for (const TraceGroup &g : m->trace_groups)
+        for (const TraceGroup &g : m->trace_groups) {
             launch_trace(m->precision, cfg, g.nn, m->sys.p, m->comp_type.p, m->comp_plane.p,
                          m->cf.p, m->cd.p, m->valid.p, P, m->C_total, m->trace_blocks.p + g.off,
                          g.count, m->need.p, m->nodes_chi(), p0, nP, m->Lbuf.p, m->total_pix, st,
-                         m->ffq(), m->work.p);
-        if (is_mixed(m->precision))
+                         m->ffq(), m->work.p, zeroed);
+            zeroed = zeroed && g.count <= 0;
+        }
+        if (is_mixed(m->precision) && m->n_trace_blocks > 0)
             launch_fix64(cfg, m->sys.p, 0, m->n_sys, m->comp_type.p, m->comp_plane.p, m->cf.p,
                          m->cd.p, m->valid.p, P, m->C_total, m->need.p, m->nodes_chi(), p0, nP,
                          m->Lbuf.p, m->total_pix, st);
@@ -1654,7 +1658,7 @@ extern "C" int lensed_loglike_plain(lensed_model *m, const double *params, int P
                          m->cd.p, m->valid.p, P, m->C_total,
                          m->trace_blocks.p + m->trace_sys_off[s], m->trace_sys_cnt[s], m->need.p,
                          m->nodes_chi(), p, 1, m->Lbuf.p, m->total_pix, st);
-            if (is_mixed(m->precision))
+            if (is_mixed(m->precision) && m->trace_sys_cnt[s] > 0)
                 launch_fix64(cfg, m->sys.p, s, 1, m->comp_type.p, m->comp_plane.p, m->cf.p,
                              m->cd.p, m->valid.p, P, m->C_total, m->need.p, m->nodes_chi(), p, 1,
                              m->Lbuf.p, m->total_pix, st);
@@ -1786,7 +1790,7 @@ extern "C" int lensed_batch_plan(lensed_model *m, int P, int *launches, int *chu
     if (m->precision == LENSED_PREC_MIXED_FF && m->cfg().ff_split && m->ffq_cnt.p)
         for (const TraceGroup &g : m->trace_groups) second += 3 * (g.nn >= 1 && g.nn <= 8);
     *launches = 3 + chunks * ((int)m->trace_groups.size() + (int)m->psf_groups.size() +
-                              (is_mixed(m->precision) ? 1 : 0) + second);
+                              (is_mixed(m->precision) && m->n_trace_blocks > 0 ? 1 : 0) + second);
     *chunk_points = m->chunk();
     return LENSED_OK;
 }
@@ -1940,7 +1944,7 @@ extern "C" int lensed_loglike_batch_noalloc(lensed_model *m, const double *param
             launch_trace(m->precision, cfg, g.nn, m->sys.p, m->comp_type.p, m->comp_plane.p, cf,
                          cd, valid, P, m->C_total, m->trace_blocks.p + g.off, g.count, m->need.p,
                          m->nodes_chi(), p0, nP, Lbuf, m->total_pix, st);
-        if (is_mixed(m->precision))
+        if (is_mixed(m->precision) && m->n_trace_blocks > 0)
             launch_fix64(cfg, m->sys.p, 0, m->n_sys, m->comp_type.p, m->comp_plane.p, cf, cd,
                          valid, P, m->C_total, m->need.p, m->nodes_chi(), p0, nP, Lbuf,
                          m->total_pix, st);
