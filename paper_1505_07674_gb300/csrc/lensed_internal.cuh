@@ -114,9 +114,23 @@ static_assert(kTileH == 32 && kTileW == 64 && kPsfThreads == 256,
 struct LaunchCfg {
     int trace_threads;  // threads per trace block, one pixel each
     int psf_sep;        // 1: PSFs of low rank run as separable passes
-    int ff_split;       // 1 (MIXED_FF): float-float re-traces in a second kernel
+    int ff_split;       // 1 (MIXED_FF): float-float re-traces in a second kernel; 2: in
+                        // launches of kSecondPassBlocks and more
     int persistent;     // 1: the trace runs as a persistent, work-queued launch
 };
+
+// Where the default (ff_split 2) takes the second pass: its three more kernels
+// cost a fixed 30 us, which the two-pixel first pass wins back in larger
+// launches.  A call in ms, in-block / second pass, by blocks of the launch:
+// 64 x 64, 5 x 5 rays: 4,096 .162/.170, 8,192 .262/.252; 200 x 200: 10,016
+// .146/.155, 20,032 .224/.220; 400 x 400: 10,000 .252/.266, 20,000 .454/.440;
+// 160 x 160, 7 x 7 rays, two lenses: 3,200 .326/.334, 6,400 .540/.531.
+constexpr long long kSecondPassBlocks = 10240;
+inline bool second_pass(LaunchCfg cfg, int nn, long long blocks)
+{
+    return nn >= 1 && nn <= 8 &&
+           (cfg.ff_split == 1 || (cfg.ff_split == 2 && blocks >= kSecondPassBlocks));
+}
 
 // One deferred float-float ray of a trace launch: lin = the pixel's index in
 // the launch's image scratch ((point - p0) * stride + pixel offset of the
@@ -170,9 +184,9 @@ void launch_prologue(const SysDev *sys, const int *comp_sys, int s0, int nS, int
 
 // a2-a5: pixel luminosities of the pixels in the block table, for points
 // p0 .. p0 + nP - 1, into Lbuf[(p - p0) * L_stride + pix_off + pix].  Every
-// system in the table has nn nodes per row of its rule.  MIXED_FF with
-// cfg.ff_split and a queue (q.cnt != nullptr): the float-float re-traces run
-// in a second kernel after the first (same results bit for bit).  zeroed: the
+// system in the table has nn nodes per row of its rule.  MIXED_FF where
+// second_pass() says so, with a queue (q.cnt != nullptr): the float-float
+// re-traces run in kernels after the first (same results bit for bit).  zeroed: the
 // prologue has zeroed the counters of q and work.
 void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const int *comp_type,
                   const int *comp_plane, const float *cf, const double *cd,

@@ -1681,8 +1681,8 @@ void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const
     } else if (precision == LENSED_PREC_MIXED_FF) {
         // the global queue needs the deferral mask, i.e. at most 8 nodes per
         // row, and 32-bit pixel indices into this launch's scratch
-        const bool split = cfg.ff_split && q.cnt && q.ent && q.val && q.pix && q.prun && nn >= 1 &&
-                           nn <= 8 &&
+        const bool split = second_pass(cfg, nn, (long long)n_blocks * nP) && q.cnt && q.ent &&
+                           q.val && q.pix && q.prun &&
                            (long long)nP * L_stride < (long long)kFfNone;
         if (split) {
             if (!zeroed) cudaMemsetAsync(q.cnt, 0, 2 * sizeof(unsigned long long), st);

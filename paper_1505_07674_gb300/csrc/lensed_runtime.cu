@@ -560,14 +560,20 @@ struct lensed_model {
     unsigned long long graph_clock = 0;
 
     // The default (no configuration chosen) is configuration 0, in MIXED_FF
-    // with the second pass (12): the same bits, and its first pass traces two
-    // pixels per thread (1,024 points of the 200x200 workload 2.64 -> 2.15 ms a
-    // call, 100 points of the 400x400 one 2.61 -> 2.30 ms).
+    // with the second pass (12) in all but small launches (kSecondPassBlocks):
+    // the same bits, and its first pass traces two pixels per thread (1,024
+    // points of the 200x200 workload 2.64 -> 2.11 ms a call, 100 points of the
+    // 400x400 one 2.61 -> 2.24 ms).
     int default_index() const
     {
         return precision == LENSED_PREC_MIXED_FF ? kBaseCandidates : 0;
     }
-    LaunchCfg cfg() const { return kCandidates[cfg_index < 0 ? default_index() : cfg_index].cfg; }
+    LaunchCfg cfg() const
+    {
+        LaunchCfg c = kCandidates[cfg_index < 0 ? default_index() : cfg_index].cfg;
+        if (cfg_index < 0 && c.ff_split) c.ff_split = 2;
+        return c;
+    }
     // points per chunk of the batched schedule (after ensure_capacity)
     int chunk() const { return chunk_limit > 0 ? std::min(chunk_P, chunk_limit) : chunk_P; }
     int n_candidates() const
@@ -1785,12 +1791,16 @@ extern "C" int lensed_batch_plan(lensed_model *m, int P, int *launches, int *chu
     if (rc) return rc;
     const int chunks = (P + m->chunk() - 1) / m->chunk();
     // a MIXED_FF second pass: three more kernels (pixel refinement, re-trace,
-    // apply) per trace group of at most 8 nodes per row
+    // apply) per trace group that takes it
     int second = 0;
-    if (m->precision == LENSED_PREC_MIXED_FF && m->cfg().ff_split && m->ffq_cnt.p)
-        for (const TraceGroup &g : m->trace_groups) second += 3 * (g.nn >= 1 && g.nn <= 8);
-    *launches = 3 + chunks * ((int)m->trace_groups.size() + (int)m->psf_groups.size() +
-                              (is_mixed(m->precision) && m->n_trace_blocks > 0 ? 1 : 0) + second);
+    if (m->precision == LENSED_PREC_MIXED_FF && m->ffq_cnt.p)
+        for (int p0 = 0; p0 < P; p0 += m->chunk())
+            for (const TraceGroup &g : m->trace_groups)
+                second += 3 * second_pass(m->cfg(), g.nn,
+                                          (long long)g.count * std::min(m->chunk(), P - p0));
+    *launches = 3 + second +
+                chunks * ((int)m->trace_groups.size() + (int)m->psf_groups.size() +
+                          (is_mixed(m->precision) && m->n_trace_blocks > 0 ? 1 : 0));
     *chunk_points = m->chunk();
     return LENSED_OK;
 }
