@@ -9,12 +9,13 @@
 //               copies; per (system, point): validity, and the image-plane
 //               priors (a source moved to theta - alpha(theta)).
 //   k_trace_rows, k_trace_rows_pq
-//               a2-a5: one thread per needed pixel; for every ray of the
+//               a2-a5: one thread per two needed pixels (lensed_pair.cuh), or
+//               per one where the block re-traces its own rays; for every ray of the
 //               quadrature rule: ray position (Eq. 14), deflection (Eq. 1),
 //               brightness at image and traced position (Eq. 2), weighted
 //               sum into the pixel luminosity (Eq. 3), in registers, starting
 //               from the once-per-model integral of the fixed lights.  The
-//               rays of a node row are traced in pairs with packed FP32
+//               rays of two pixels, or two of a node row, share packed FP32
 //               instructions (lensed_vec2.cuh).  _pq: the same work as a
 //               persistent grid taking (trace block, point) items from a
 //               counter.  MIXED_FF re-traces the rays near a source centre
@@ -31,7 +32,8 @@
 //               with the PSF row and the image row segment held in
 //               registers (or, for a PSF of rank <= 3, a row pass and a
 //               column pass per separable term); then the masked chi^2 of the
-//               tile (Eq. 17) as a warp-shuffle tree in FP64, or the image.
+//               tile (Eq. 17), float pairs through a warp and FP64 beyond, or
+//               the image.
 //   k_finalize  a7: loglike = -1/2 sum of the tile partials, fixed order.
 //   k_error_image
 //               the Gauss-Kronrod error estimate |L_K - L_G| of a render.
@@ -1733,7 +1735,10 @@ void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const
 // in it, so the rays are first sorted and the FP64 ones run on warps of their
 // own; and where a launch has fewer (system, point) pairs than the GPU has
 // SMs, kFixSlices blocks share a pair's pixels.  Trace stage 736 -> 718 us
-// (64x64, 1,000 points), 1,655 -> 1,644 us (200x200, 1,024 points).
+// (64x64, 1,000 points), 1,655 -> 1,644 us (200x200, 1,024 points).  What
+// all four warps computed alike in FP64 (half of a block's FP64 instructions)
+// is done by one, and rays known to need no FP64 issue none: 713 -> 699,
+// 1,647 -> 1,635 us; two points of 160x160 with two lenses, 91 -> 74 us.
 
 // Does the MIXED rule evaluate an SIE in FP64 for ray (a, b) of pixel (jc, ic)?
 // (decided in FP32 unless the ray is within rounding of the disc's edge)
@@ -1758,9 +1763,10 @@ __device__ __forceinline__ bool ray_wants_f64(const TraceSmem &sm, const SysDev 
     return false;
 }
 
-// Brightness of ray (a, b) of pixel (i, j) under the MIXED rule.
+// Brightness of ray (a, b) of pixel (i, j) under the MIXED rule; w64: it takes
+// some SIE in FP64 (ray_wants_f64; the others need no FP64 instruction).
 __device__ float ray_mixed(const TraceSmem &sm, const SysDev &S, int i, int j, int a, int b,
-                          bool ff)
+                          bool ff, bool w64)
 {
     const int ncomp = S.ncomp;
     const float jc = (float)j - S.cx, ic = (float)i - S.cy;
@@ -1776,8 +1782,8 @@ __device__ float ray_mixed(const TraceSmem &sm, const SysDev &S, int i, int j, i
             const int t = sm.type[c];
             if (t == LENSED_SIE) {
                 const double *cd = sm.cd + c * kNC;
-                bool use64 = cd[17] != 0.0;
-                if (!use64) {
+                bool use64 = w64 && cc[17] != 0.f;
+                if (w64 && !use64) {
                     const double dx = (double)jc * S.hd + sm.ud[a] - cd[0];
                     const double dy = (double)ic * S.hd + sm.ud[b] - cd[1];
                     use64 = dx * dx + dy * dy < cd[18];
@@ -1853,7 +1859,7 @@ __device__ void fix_pixels(const TraceSmem &sm, const SysDev &S, const int *s_pi
             if (e >= n64 && e < pad) continue;
             const int t = s_list[e < n64 ? e : n64 + e - pad], pix = s_pix[b0 + t / nr], r = t % nr;
             const int i = pix / nx, j = pix - (pix / nx) * nx;
-            s_ray[t] = ray_mixed(sm, S, i, j, r % nn, r / nn, ff);
+            s_ray[t] = ray_mixed(sm, S, i, j, r % nn, r / nn, ff, e < n64);
         }
         __syncthreads();
         chain_wait();
@@ -1882,6 +1888,7 @@ __global__ void __launch_bounds__(128)
     __shared__ int s_pix[kFixRays];
     __shared__ unsigned short s_list[kFixRays];
     __shared__ int s_n, s_m[2];
+    __shared__ int4 s_box[LENSED_MAX_COMPONENTS];  // first and last column, row of a disc
     const int slice = blockIdx.z, slices = gridDim.z;
     const int s = s0 + blockIdx.x;
     const int p = p0 + blockIdx.y;
@@ -1898,7 +1905,7 @@ __global__ void __launch_bounds__(128)
     const float *pre = (nodes.pre_f && S.pre_off >= 0) ? nodes.pre_f + S.pre_off : nullptr;
     bool whole = false;
     for (int c = 0; c < ncomp; ++c)
-        if (sm.type[c] == LENSED_SIE && sm.cd[c * kNC + 17] != 0.0) whole = true;
+        if (sm.type[c] == LENSED_SIE && sm.cf[c * kNC + 17] != 0.f) whole = true;
     if (whole) {
         // every listed pixel, in slices
         const int n = need ? S.n_need : S.npix;
@@ -1913,17 +1920,26 @@ __global__ void __launch_bounds__(128)
         chain_wait();
         return;
     }
-    // core discs, one SIE after the other; a pixel already covered by an
-    // earlier SIE's disc is skipped so every pixel is written once
+    // the boxes of the core discs, one thread per component: computed by every
+    // thread they were four FP64 quotients and a root on each of the four warps
+    if ((int)threadIdx.x < ncomp) {
+        int4 box = make_int4(0, -1, 0, -1);
+        const double *cc = sm.cd + threadIdx.x * kNC;
+        if (sm.type[threadIdx.x] == LENSED_SIE && cc[18] > 0.0) {
+            const double r = sqrt(cc[18]);
+            box.x = max(0, (int)floor((cc[0] - r) / S.hd + S.cx - 1.0));
+            box.y = min(nx - 1, (int)ceil((cc[0] + r) / S.hd + S.cx + 1.0));
+            box.z = max(0, (int)floor((cc[1] - r) / S.hd + S.cy - 1.0));
+            box.w = min(ny - 1, (int)ceil((cc[1] + r) / S.hd + S.cy + 1.0));
+        }
+        s_box[threadIdx.x] = box;
+    }
+    __syncthreads();
+    // one SIE after the other; a pixel already covered by an earlier SIE's
+    // disc is skipped so every pixel is written once
     for (int c = 0; c < ncomp; ++c) {
-        if (sm.type[c] != LENSED_SIE) continue;
         const double *cc = sm.cd + c * kNC;
-        const double r = sqrt(cc[18]);
-        if (!(r > 0.0)) continue;
-        const int j0 = max(0, (int)floor((cc[0] - r) / S.hd + S.cx - 1.0));
-        const int j1 = min(nx - 1, (int)ceil((cc[0] + r) / S.hd + S.cx + 1.0));
-        const int i0 = max(0, (int)floor((cc[1] - r) / S.hd + S.cy - 1.0));
-        const int i1 = min(ny - 1, (int)ceil((cc[1] + r) / S.hd + S.cy + 1.0));
+        const int j0 = s_box[c].x, j1 = s_box[c].y, i0 = s_box[c].z, i1 = s_box[c].w;
         if (j1 < j0 || i1 < i0) continue;
         const int bw = j1 - j0 + 1, nbox = bw * (i1 - i0 + 1);
         for (int q0 = 0; q0 < nbox; q0 += kFixRays) {
