@@ -1555,7 +1555,8 @@ __global__ void __launch_bounds__(kFfThreads)
 
 // Each refined pixel's re-traced rays are added, in ray order, to the sum
 // k_refine_ff stored: one thread per pixel record, its rays a contiguous
-// slice of the queue.
+// slice of the queue.  Bound by the latency of its chain of loads, so the ones
+// that do not depend on each other are issued together.
 __global__ void k_apply_ff(const SysDev *__restrict__ sys, NodeTables nodes,
                            float *__restrict__ Lbuf, FfQueue fq)
 {
@@ -1563,11 +1564,12 @@ __global__ void k_apply_ff(const SysDev *__restrict__ sys, NodeTables nodes,
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x) {
         const uint2 run = fq.prun[e];
-        if (run.y == 0u) continue;
         const FfEntry R = fq.pix[e];
+        if (run.y == 0u) continue;
         const SysDev &S = sys[R.sr];
         const float *w = nodes.w + S.w2_off;
         float acc = Lbuf[R.lin];
+#pragma unroll 4
         for (unsigned k = 0; k < run.y; ++k) {
             const unsigned sr = fq.ent[run.x + k].sr;
             acc = fmaf(w[(sr >> 3 & 7u) * (unsigned)S.nn + (sr & 7u)], fq.val[run.x + k], acc);
@@ -1665,6 +1667,25 @@ static void trace_rows_dispatch(int nn, int threads, const SysDev *sys, const in
 #undef LENSED_ROWS
 }
 
+// Grid of a second-pass kernel: as many blocks as fit the chip at once, times
+// waves, each striding over its share of the queue.  Eight blocks per SM,
+// whatever fits, gave k_refine_ff (5 resident at 94 registers) a second wave
+// that was 3/5 full, and k_apply_ff half of the loads in flight that it can
+// have: 749 -> 744 us a call (64x64, 1,000 points).  k_retrace_ff takes four
+// waves: its rays' paths differ in length, and with fixed shares warps ran out
+// of work early (38 % of the warp slots used of 50 % resident); 746 -> 729 us,
+// 1.861 -> 1.849 ms (200x200, 1,024 points).  Sixteen cost a small launch (32
+// points of 200x200) 8 us for blocks that find nothing to do.
+template <class... K>
+static unsigned resident_grid(void (*kernel)(K...), unsigned waves = 1)
+{
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, kFfThreads, 0) !=
+        cudaSuccess)
+        per_sm = 8;
+    return waves * (unsigned)(std::max(1, g_sm_count) * std::max(1, per_sm));
+}
+
 void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const int *comp_type,
                   const int *comp_plane, const float *cf, const double *cd,
                   const unsigned char *valid, int P, int C_total, const TraceBlock *blocks,
@@ -1691,10 +1712,9 @@ void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const
             trace_rows_dispatch<LENSED_PREC_MIXED_FF, true>(
                 nn, cfg.trace_threads, sys, comp_type, comp_plane, cf, cd, valid, P, C_total,
                 blocks, n_blocks, need, nodes, p0, nP, Lbuf, L_stride, st, q, work);
-            const unsigned grid = (unsigned)std::max(1, g_sm_count) * 8;
 #define LENSED_REFINE(GG)                                                                     \
-    k_refine_ff<GG><<<grid, kFfThreads, 0, st>>>(sys, comp_type, comp_plane, cf, C_total, nodes, \
-                                                 p0, (unsigned)L_stride, (float *)Lbuf, q)
+    k_refine_ff<GG><<<resident_grid(k_refine_ff<GG>), kFfThreads, 0, st>>>(                    \
+        sys, comp_type, comp_plane, cf, C_total, nodes, p0, (unsigned)L_stride, (float *)Lbuf, q)
             switch (nn) {
             case 1: LENSED_REFINE(1); break;
             case 2: LENSED_REFINE(2); break;
@@ -1706,9 +1726,9 @@ void launch_trace(int precision, LaunchCfg cfg, int nn, const SysDev *sys, const
             default: LENSED_REFINE(8); break;
             }
 #undef LENSED_REFINE
-            k_retrace_ff<<<grid, kFfThreads, 0, st>>>(sys, comp_type, comp_plane, cf, C_total,
-                                                     nodes, p0, (unsigned)L_stride, q);
-            k_apply_ff<<<grid, kFfThreads, 0, st>>>(sys, nodes, (float *)Lbuf, q);
+            k_retrace_ff<<<resident_grid(k_retrace_ff, 4), kFfThreads, 0, st>>>(
+                sys, comp_type, comp_plane, cf, C_total, nodes, p0, (unsigned)L_stride, q);
+            k_apply_ff<<<resident_grid(k_apply_ff), kFfThreads, 0, st>>>(sys, nodes, (float *)Lbuf, q);
         } else {
             trace_rows_dispatch<LENSED_PREC_MIXED_FF, false>(
                 nn, cfg.trace_threads, sys, comp_type, comp_plane, cf, cd, valid, P, C_total,
