@@ -443,7 +443,7 @@ def run_mlp(args):
                          "peak": peak, "unit": "TFLOP/s",
                          "frac": f_flops / (f_ms * 1e-3) / 1e12 / peak,
                          "peak_source": f"bf16_tflops ({pk_src})",
-                         "kernel": "k_gemm_tc (tcgen05.mma, TMEM accumulators)"},
+                         "kernel": "k_forward (tcgen05.mma, TMEM accumulators)"},
             "clocks": clocks}
     print(json.dumps(line), flush=True)
     return 0

@@ -303,7 +303,7 @@ int lensed_loglike_batch_noalloc(lensed_model *m, const double *params, int P,
  * the trace as one CTA per (trace block, point) or as a persistent,
  * work-queued launch whose resident CTAs take those items from a counter;
  * for LENSED_PREC_MIXED_FF also whether the float-float re-traces run inside
- * the trace blocks or in a second kernel) on a batch of P points drawn
+ * the trace blocks or in a second pass) on a batch of P points drawn
  * inside the given DEVICE parameter array (same layout as
  * lensed_loglike_batch) and keep the fastest for later calls; then, with
  * that configuration, time whole scratch chunks against chunks sized to half
@@ -342,7 +342,8 @@ int lensed_eval_sie_trig(const float *n, const float *d, long long count, float 
  * same three with separable passes; 6-11 = 0-5 with the trace as a
  * persistent, work-queued launch.  LENSED_PREC_MIXED_FF: n = 24, and
  * 12 + k runs configuration k with the float-float re-traces in a second
- * kernel. */
+ * pass.  The default is 0; for LENSED_PREC_MIXED_FF 12, with the re-traces
+ * inside the trace blocks in launches too small for a second pass to pay. */
 int lensed_set_config(lensed_model *m, int index);
 
 /* Points per scratch chunk of the batched schedule (a8; the paper has no
