@@ -201,7 +201,7 @@ void init_kernel_attributes();
 
 // MIXED only: recompute, with the FP64 SIE, the pixels of each (system,
 // point) that the MIXED rule assigns to FP64 (after launch_trace wrote
-// their FP32 values; it follows a trace launch on st, beside which it starts).
+// their FP32 values).
 // need == nullptr: every pixel of the systems (render).
 void launch_fix64(LaunchCfg cfg, const SysDev *sys, int s0, int nS, const int *comp_type,
                   const int *comp_plane, const float *cf, const double *cd,

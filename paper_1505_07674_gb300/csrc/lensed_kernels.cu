@@ -56,7 +56,8 @@ namespace lensed {
 // the kernel before it in the stream still runs (once all of that one's
 // blocks have started and called chain_next, or exited), so its launch and
 // prologue cost no gap.  Every block calls chain_wait before it touches
-// anything that an earlier kernel of the stream reads or writes: that returns
+// anything that an earlier kernel of the stream, the one before or any other,
+// reads or writes: that returns
 // when the earlier kernel has completed, which by the same rule has waited for
 // the one before it.  Eight points of a 64 x 64 image, a call: 87 us launch by
 // launch, 69 us so; a render with its error map: 283 and 212 us.  The kernels
@@ -1882,7 +1883,6 @@ __device__ void fix_pixels(const TraceSmem &sm, const SysDev &S, const int *s_pi
             s_ray[t] = ray_mixed(sm, S, i, j, r % nn, r / nn, ff, e < n64);
         }
         __syncthreads();
-        chain_wait();
         for (int k = threadIdx.x; k < m; k += blockDim.x) {
             float acc = pre ? pre[s_pix[b0 + k]] : 0.f;
             for (int r = 0; r < nr; ++r) acc = fmaf(sm.w[r], s_ray[k * nr + r], acc);
@@ -1899,9 +1899,9 @@ __global__ void __launch_bounds__(128)
                   int C_total, const int *__restrict__ need, NodeTables nodes, int p0,
                   float *__restrict__ Lbuf, long long L_stride)
 {
-    // the constants are there (the trace kernel waited for the prologue before
-    // it let this one start), so the rays are computed beside the trace; only
-    // writing pixels has to wait for it
+    // (before the constants, too: what the prologue wrote is promised to a grid
+    // that waits itself, not to one that an intermediate grid let start)
+    chain_wait();
     chain_next();
     __shared__ __align__(16) TraceSmem sm;
     __shared__ float s_ray[kFixRays];
@@ -1912,10 +1912,7 @@ __global__ void __launch_bounds__(128)
     const int slice = blockIdx.z, slices = gridDim.z;
     const int s = s0 + blockIdx.x;
     const int p = p0 + blockIdx.y;
-    if (!valid[(size_t)s * P + p]) {
-        chain_wait();
-        return;
-    }
+    if (!valid[(size_t)s * P + p]) return;
     const SysDev &S = sys[s];
     const size_t cbase = ((size_t)p * C_total + S.comp_off) * kNC;
     stage_point(sm, S, comp_type, comp_plane, cf, cd, cbase, true, false, nodes);
@@ -1937,7 +1934,6 @@ __global__ void __launch_bounds__(128)
             __syncthreads();
             fix_pixels(sm, S, s_pix, m, s_ray, s_list, s_m, L, pre, nodes.ff != 0);
         }
-        chain_wait();
         return;
     }
     // the boxes of the core discs, one thread per component: computed by every
@@ -1983,7 +1979,6 @@ __global__ void __launch_bounds__(128)
             fix_pixels(sm, S, s_pix, n, s_ray, s_list, s_m, L, pre, nodes.ff != 0);
         }
     }
-    chain_wait();
 }
 
 void launch_fix64(LaunchCfg cfg, const SysDev *sys, int s0, int nS, const int *comp_type,
