@@ -32,8 +32,7 @@
 //               with the PSF row and the image row segment held in
 //               registers (or, for a PSF of rank <= 3, a row pass and a
 //               column pass per separable term); then the masked chi^2 of the
-//               tile (Eq. 17), float pairs through a warp and FP64 beyond, or
-//               the image.
+//               tile (Eq. 17), summed in FP64, or the image.
 //   k_finalize  a7: loglike = -1/2 sum of the tile partials, fixed order.
 //   k_error_image
 //               the Gauss-Kronrod error estimate |L_K - L_G| of a render.
@@ -2006,54 +2005,6 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
-// Sum of non-negative float terms as an unevaluated pair of floats, sum +
-// rest: Knuth's two-sum keeps every addition's rounding error, and the errors
-// are summed beside it, so n terms come out with a relative error of about
-// n 2^-47.  FP64 runs at 1/64 of the FP32 rate here: converting and adding
-// each of a thread's 8 chi^2 terms and 5 shuffle steps in FP64 kept the FP64
-// unit 45 % busy in k_psf_sep; PSF stage 526 -> 485 us on the uneven systems,
-// 41 -> 37 us (64x64, 1,000 points), 248 -> 242 us (200x200, 1,024 points).
-// An infinite or NaN sum is carried by `sum` alone.
-struct PairSum {
-    float sum = 0.f, rest = 0.f;
-    __device__ __forceinline__ void add(float t)
-    {
-        const float s = __fadd_rn(sum, t), b = __fsub_rn(s, sum);
-        rest = __fadd_rn(rest, __fadd_rn(__fsub_rn(sum, __fsub_rn(s, b)), __fsub_rn(t, b)));
-        sum = s;
-    }
-    __device__ __forceinline__ double value() const
-    {
-        return isfinite(sum) ? (double)sum + (double)rest : (double)sum;
-    }
-};
-__device__ __forceinline__ PairSum warp_sum(PairSum v)
-{
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        const float s = __shfl_xor_sync(0xffffffffu, v.sum, o);
-        const float r = __shfl_xor_sync(0xffffffffu, v.rest, o);
-        v.add(s);
-        v.rest = __fadd_rn(v.rest, r);
-    }
-    return v;
-}
-// chi^2 of a thread: float terms in a pair, double terms (FP64 mode) as they are
-template <typename T>
-struct Chi;
-template <>
-struct Chi<float> {
-    PairSum v;
-    __device__ __forceinline__ void add(float t) { v.add(t); }
-    __device__ __forceinline__ double warp() const { return warp_sum(v).value(); }
-};
-template <>
-struct Chi<double> {
-    double v = 0.0;
-    __device__ __forceinline__ void add(double t) { v += t; }
-    __device__ __forceinline__ double warp() const { return warp_sum(v); }
-};
-
 static __host__ __device__ __forceinline__ int psf_row_stride(int q)
 {
     // row of the staged tile: kTileW + 2q values, rounded up to a multiple of 4
@@ -2226,7 +2177,7 @@ __global__ void __launch_bounds__(kPsfThreads)
     }
 
     if (partial) {
-        Chi<T> chi;
+        double chi = 0.0;
         if (live && i < ny) {
 #pragma unroll
             for (int o = 0; o < kOutPerThread; ++o) {
@@ -2235,16 +2186,18 @@ __global__ void __launch_bounds__(kPsfThreads)
                     const size_t pix = S.pix_off + (size_t)i * nx + j;
                     const T w = weight[pix];
                     if (w > T(0)) {
-                        // one product per pixel in the working precision
+                        // one product per pixel in the working precision,
+                        // summed in FP64: the sum of a warp's float products
+                        // may lie beyond the largest float
                         const T r = data[pix] - acc[o];
-                        chi.add(w * r * r);
+                        chi += (double)(w * r * r);
                     }
                 }
             }
         }
         // warp-shuffle tree, then across the 8 warps in fixed order
         __shared__ double s_red[kPsfThreads / 32];
-        const double total = live ? chi.warp() : 0.0;  // (live is the same for the whole warp)
+        const double total = live ? warp_sum(chi) : 0.0;  // (live is the same for the whole warp)
         if (lane == 0) s_red[warp] = total;
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -2432,16 +2385,16 @@ __global__ void __launch_bounds__(kPsfThreads, 4)
     }
 
     if (partial) {
-        Chi<float> chi;
+        double chi = 0.0;
 #pragma unroll
         for (int o = 0; o < 2 * kR; ++o) {
             if (wv[o] > 0.f) {
                 const float r = dv[o] - (o & 1 ? acc[o >> 1].y : acc[o >> 1].x);
-                chi.add(wv[o] * r * r);
+                chi += (double)(wv[o] * r * r);
             }
         }
         __shared__ double s_red[kPsfThreads / 32];
-        const double total = live ? chi.warp() : 0.0;  // (live is the same for the whole warp)
+        const double total = live ? warp_sum(chi) : 0.0;  // (live is the same for the whole warp)
         if (lane == 0) s_red[warp] = total;
         __syncthreads();
         if (threadIdx.x == 0) {

@@ -68,3 +68,27 @@ def test_silu_derivative_of_very_negative_values_vanishes(x):
     # silu'(z) ~ z exp(z): at most 6e-25 in size
     assert abs(g[o_b1]) <= 1e-24, g[o_b1]
     assert abs(g[0]) <= 1e-24 * max(1.0, abs(x)) and np.isfinite(g).all()
+
+
+@pytest.mark.parametrize("precision,config", [("fp32", 0), ("fp32", 3), ("mixed_ff", 0), ("mixed_ff", 12),
+                                              ("fp64", 0)])
+def test_chi2_beyond_the_largest_float(precision, config):
+    # every pixel's squared residual fits a float, the sum of a warp's does not.
+    # The source is too faint for a float; per term the rounding of the data and
+    # of two products (4 x 2^-24), the sum in FP64: 1e-6
+    from paper_1505_07674_gb300 import lensed as LZ
+    from workloads import component, fixed, free
+    comps = [component("gauss", "source", [free(0), fixed(0.0), fixed(0.3), fixed(1000.0), fixed(0.7),
+                                           fixed(30.0)])]
+    ny, nx = 40, 70
+    psf = np.outer([1.0, 2.0, 1.0], [1.0, 3.0, 1.0])
+    spec = {"nx": nx, "ny": ny, "h": 0.05, "rule": ("gl", 2), "psf": psf, "mask": None, "zeropoint": 0.0,
+            "components": comps, "n_params": 1}
+    rng = np.random.default_rng(2)
+    data = rng.uniform(0.9e19, 1.8e19, (ny, nx))
+    m = LZ.Model(spec, {"data": data, "variance": np.ones((ny, nx))}, precision=precision)
+    m.set_config(config)
+    got = m.loglike_batch(np.array([[0.0], [0.1]])).cpu().numpy()
+    m.close()
+    want = -0.5 * np.sum(data * data)
+    assert np.all(np.abs(got - want) <= 1e-6 * abs(want)), got
