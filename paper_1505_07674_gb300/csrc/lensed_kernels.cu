@@ -63,7 +63,7 @@ namespace lensed {
 // of a second pass are launched without it: their grids are sized to the whole
 // chip, and started as a trace drains, the first idle multiprocessors would
 // take most of their blocks (1,024 points of a 200 x 200 image, trace stage:
-// 1.65 ms so, 1.68 ms chained).
+// 1.65 ms so, 1.68 ms chained); so is the fix-up, but for the smallest launches.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next()
 {
@@ -1852,6 +1852,13 @@ __device__ __forceinline__ bool pixel_near(const SysDev &S, int i, int j, double
 
 constexpr int kFixRays = 1024;  // ray contributions staged per batch
 constexpr int kFixSlices = 8;   // blocks of a (system, point) in a small launch
+// Chained behind the trace up to this many blocks.  More are launched once it
+// has finished: started while it drains, the first idle multiprocessors took
+// most of them, and their FP64 units most of the work.  A call of 24 x 24
+// pixels in us, chained / launched after: 256 points, 16 x 16 rays, two lenses
+// 941 / 637; 77 points, 5 x 5 rays, one lens 64 / 52.  A render (8 blocks) of
+// 64 x 64 pixels 44 / 46.
+constexpr long long kFixChained = 32;
 
 // Recompute the pixels of s_pix[0..n) (batches of kFixRays / (nn*nn)).
 __device__ void fix_pixels(const TraceSmem &sm, const SysDev &S, const int *s_pix, int n,
@@ -1991,8 +1998,12 @@ void launch_fix64(LaunchCfg cfg, const SysDev *sys, int s0, int nS, const int *c
     const long long pairs = (long long)nS * nP;
     const unsigned slices = pairs * 2 > std::max(1, g_sm_count) ? 1u : (unsigned)kFixSlices;
     dim3 grid((unsigned)nS, (unsigned)nP, slices);
-    chain(k_trace_fix64, grid, 128, 0, st, sys, s0, comp_type, comp_plane, cf, cd, valid, P,
-          C_total, need, nodes, p0, (float *)Lbuf, L_stride);
+    if (pairs * slices <= kFixChained)
+        chain(k_trace_fix64, grid, 128, 0, st, sys, s0, comp_type, comp_plane, cf, cd, valid, P,
+              C_total, need, nodes, p0, (float *)Lbuf, L_stride);
+    else
+        k_trace_fix64<<<grid, 128, 0, st>>>(sys, s0, comp_type, comp_plane, cf, cd, valid, P,
+                                            C_total, need, nodes, p0, (float *)Lbuf, L_stride);
 }
 
 // ---------------------------------------------------------------------------
