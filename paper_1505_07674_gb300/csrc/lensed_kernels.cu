@@ -1394,10 +1394,17 @@ __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs
 
 // The same work as a persistent, work-queued launch: a grid sized to the
 // resident CTAs of the GPU takes (trace block, point) items, point-major,
-// kPqGrab at a time from the counter *work (zeroed before the launch) until
+// `grab` at a time from the counter *work (zeroed before the launch) until
 // n_items are done, staging a point's constants only when the system or the
 // point changes.
-constexpr int kPqGrab = 4;
+//
+// They are taken kPqGrab at a time where every CTA gets two such turns, fewer
+// in smaller launches: a CTA of the two-pixel form has half the threads and
+// each twice the pixels, and four items in a row left most of the chip idle.
+// A call in us, two lenses, FP32, always four / by this rule: 16 points of 160 x
+// 160 pixels, 7 x 7 rays 358 / 173, 16 x 16 rays 1,688 / 760; one point of 64 x 64
+// pixels, 7 x 7 rays 148 / 58.
+constexpr unsigned kPqGrab = 4;  // (the turns are powers of two)
 template <int MODE, int G, bool EXACT, bool GQ>
 __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs<MODE, GQ> ? 6 : 0)
     k_trace_rows_pq(const SysDev *__restrict__ sys, const int *__restrict__ comp_type,
@@ -1406,25 +1413,25 @@ __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs
                     int C_total, const TraceBlock *__restrict__ blocks,
                     const int *__restrict__ need, NodeTables nodes, int p0,
                     float *__restrict__ Lbuf, long long L_stride, FfQueue fq, int n_blocks,
-                    unsigned n_items, unsigned long long *__restrict__ work)
+                    unsigned n_items, unsigned grab, unsigned long long *__restrict__ work)
 {
     chain_wait();
     chain_next();
     __shared__ unsigned s_item;
     __shared__ __align__(16) std::conditional_t<kTracePairs<MODE, GQ>, PairSmem, char> sm;
     for (;;) {
-        if (threadIdx.x == 0) s_item = (unsigned)atomicAdd(work, (unsigned long long)kPqGrab);
+        if (threadIdx.x == 0) s_item = (unsigned)atomicAdd(work, (unsigned long long)grab);
         __syncthreads();
         const unsigned first = s_item;
         __syncthreads();  // read by all before thread 0 takes the next ones
         if (first >= n_items) return;
-        const unsigned last = min(first + (unsigned)kPqGrab, n_items);
+        const unsigned last = min(first + grab, n_items);
 #pragma unroll 1
         for (unsigned item = first; item < last; ++item) {
             const unsigned q = item / (unsigned)n_blocks;
             const TraceBlock tb = blocks[item - q * (unsigned)n_blocks];
             // (a system's blocks follow one another from pixel 0 on)
-            const bool stage = item % (unsigned)kPqGrab == 0u || tb.start == 0;
+            const bool stage = (item & (grab - 1u)) == 0u || tb.start == 0;
             if constexpr (kTracePairs<MODE, GQ>)
                 pair_item<G, EXACT, GQ>(sm, sys, comp_type, comp_plane, cf, valid, P, C_total, need,
                                         nodes, p0, Lbuf, L_stride, fq, tb, p0 + (int)q, stage);
@@ -1635,9 +1642,11 @@ static void trace_rows_t(int threads, const SysDev *sys, const int *comp_type,
                                                   threads, 0);
     const long long want = (long long)std::max(g_sm_count, 1) * std::max(per_sm, 1);
     const unsigned grid = (unsigned)std::max(1LL, std::min(want, n_items));
+    unsigned grab = kPqGrab;
+    while (grab > 1u && n_items < 2 * grab * want) grab /= 2u;
     chain(k_trace_rows_pq<MODE, G, EXACT, GQ>, grid, threads, 0, st, sys, comp_type, comp_plane,
           cf, cd, valid, P, C_total, blocks, need, nodes, p0, (float *)Lbuf, L_stride, fq,
-          n_blocks, (unsigned)n_items, work);
+          n_blocks, (unsigned)n_items, grab, work);
 }
 
 // GQ: the launch has a global float-float queue (MIXED_FF, at most 8 nodes per row)
