@@ -379,9 +379,20 @@ __device__ __forceinline__ void pair_pixels(const PairSmem &sm, const SysDev &S,
     for (int b = 0; b < nn; ++b) {
         const float2 y = vadd(yc, sp(sm.u[b]));
         if constexpr (EXACT) {
-            for (int a0 = 0; a0 + C1 < NN; a0 += C1)
-                pair_row<C1, false, FLAG, false>(sm, nn, a0, w, xc, y, acc, near);
-            pair_row<CL, false, FLAG, (NN & 1) != 0>(sm, nn, NN - CL, w, xc, y, acc, near);
+            if constexpr (NN == 8) {
+                // the two chunks of 4 share one copy of the code, the largest of
+                // all: inlined twice it was slower than the one-pixel form with
+                // several lenses (FP32, 91 points of 160 x 160 pixels, two lenses:
+                // 1,025 us one pixel a thread, 1,074 with two copies, 1,000 with
+                // one; one lens: 530, 491 and 505)
+#pragma unroll 1
+                for (int a0 = 0; a0 < NN; a0 += C1)
+                    pair_row<C1, false, FLAG, false>(sm, nn, a0, w, xc, y, acc, near);
+            } else {
+                for (int a0 = 0; a0 + C1 < NN; a0 += C1)
+                    pair_row<C1, false, FLAG, false>(sm, nn, a0, w, xc, y, acc, near);
+                pair_row<CL, false, FLAG, (NN & 1) != 0>(sm, nn, NN - CL, w, xc, y, acc, near);
+            }
             w += kPairW;
         } else {
             for (int a0 = 0; a0 < nn; a0 += C1)
