@@ -1217,6 +1217,15 @@ __device__ __forceinline__ float pixel_rays(const KC &kc, const SysDev &S, int n
 // has pixels.  MIXED_FF with in-block re-traces keeps one pixel per thread.
 template <int MODE, bool GQ>
 constexpr bool kTracePairs = MODE != LENSED_PREC_MIXED_FF || GQ;
+// Resident CTAs of 128 threads that the two-pixel kernels are compiled for: 6
+// (80 registers), and 5 (96) for the rows that spilled most at 80: 7 nodes
+// (chunks of 4 and 3 rays, both in the code) and guarded rows.  FP32,
+// two lenses, us a call, 6 / 5: one point of 64 x 64 pixels, 16 x 16 rays 175 /
+// 152, 11 x 11 103 / 91, 7 x 7 58 / 56; 22 points of 160 x 160, 16 x 16 rays 1,031 /
+// 1,024; 119 points, 7 x 7, work-queued 1,092 / 1,051.  Rows of 4 (a few bytes
+// spilled) are 2 % slower at 5.
+template <int G, bool EXACT>
+constexpr int kPairBlocks = EXACT && G != 7 ? 6 : 5;
 
 // trace_item for two pixels per thread: items start + t and start + t +
 // blockDim.x of the block.  Lanes without an item trace the block's last one
@@ -1370,7 +1379,7 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
 }
 
 template <int MODE, int G, bool EXACT, bool GQ>
-__global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs<MODE, GQ> ? 6 : 0)
+__global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs<MODE, GQ> ? kPairBlocks<G, EXACT> : 0)
     k_trace_rows(const SysDev *__restrict__ sys, const int *__restrict__ comp_type,
                  const int *__restrict__ comp_plane, const float *__restrict__ cf,
                  const double *__restrict__ cd, const unsigned char *__restrict__ valid, int P,
@@ -1406,7 +1415,7 @@ __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs
 // pixels, 7 x 7 rays 148 / 58.
 constexpr unsigned kPqGrab = 4;  // (the turns are powers of two)
 template <int MODE, int G, bool EXACT, bool GQ>
-__global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs<MODE, GQ> ? 6 : 0)
+__global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs<MODE, GQ> ? kPairBlocks<G, EXACT> : 0)
     k_trace_rows_pq(const SysDev *__restrict__ sys, const int *__restrict__ comp_type,
                     const int *__restrict__ comp_plane, const float *__restrict__ cf,
                     const double *__restrict__ cd, const unsigned char *__restrict__ valid, int P,
