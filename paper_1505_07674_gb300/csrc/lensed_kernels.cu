@@ -195,7 +195,7 @@ __device__ __forceinline__ void sersic_b_lookup(double n, const double *__restri
 // A serial chain of FP64 functions on a unit that takes 16 cycles per warp
 // instruction, so its time is the chain's length: a CTA is one warp of one
 // component (lanes are points: no branch of another type's functions, and
-// the chains of different components run on different SMs), and the
+// the chains of different components run on different SMs), and a Sersic
 // profile's normalisation comes from a table instead of pow, lgamma and
 // three logarithms.  Prologue of a call 33 -> 20 us (8 points, 3 components),
 // 42 -> 24 us (1,024 points, 4), 51 -> 33 us (128 points, 8, an image prior).
@@ -310,9 +310,8 @@ __global__ void __launch_bounds__(kPrologueThreads) k_prologue_comp(const SysDev
         // 15 kind, 16 x0_lo, 17 y0_lo.  rho^2 = (q u^2 + v^2/q)/r^2; Sersic t = B rho^(2 p2) with
         // B = b_n log2(e), p2 = 1/(2n); Gaussian (r = sqrt(2) sigma) t =
         // B rho^2 with B = log2(e); I = A 2^-t with A = I_0 h^2.
-        // F = 10^(-0.4 (mag - zp)) enters by its logarithm
+        // Flux F = 10^(-0.4 (mag - zp)).
         const double r = v[2];
-        const double lF = -0.4 * M_LN10 * (v[3] - zeropoint);
         double n = 4.0, q, pa;
         if (type == LENSED_SERSIC) { n = v[4]; q = v[5]; pa = v[6]; }
         else { q = v[4]; pa = v[5]; }
@@ -335,10 +334,14 @@ __global__ void __launch_bounds__(kPrologueThreads) k_prologue_comp(const SysDev
             o[7] = 1.0 / (q * r2);
             o[10] = 1.0;
             o[11] = 1.4426950408889634;  // log2(e)
-            o[13] = exp(lF) / (M_PI * r2) * hd * hd;
+            // (pow: exp of the natural logarithm of F would amplify the rounding
+            // of that to twice the error)
+            const double F = pow(10.0, -0.4 * (v[3] - zeropoint));
+            o[13] = F / (M_PI * r2) * hd * hd;
             o[15] = kKindGauss;
         } else if (ok) {
             // I_0 = F b^(2n) / (2 pi n r^2 Gamma(2n)), in logs
+            const double lF = -0.4 * M_LN10 * (v[3] - zeropoint);
             double bn, g;
             sersic_b_lookup(n, bn_table, bn, g);
             const double ir2 = 1.0 / (r * r);

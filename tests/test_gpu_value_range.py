@@ -92,3 +92,28 @@ def test_chi2_beyond_the_largest_float(precision, config):
     m.close()
     want = -0.5 * np.sum(data * data)
     assert np.all(np.abs(got - want) <= 1e-6 * abs(want)), got
+
+
+def test_gaussian_flux_keeps_its_precision():
+    # one pixel of side 1 with one ray at the centre of a Gaussian: in 64 bits
+    # -2 loglike is the square of F / (2 pi sigma^2), so the ratio to magnitude
+    # 0 is F^2 = 10^(-0.8 mag).  With u = 2^-53 the exponent -0.4 mag of the
+    # power carries 1.5 u (the constant and the product), ln 10 |0.4 mag| times
+    # that in F; the power itself 2 ulp (4 u), the quotient u; F squared doubles
+    # it, and the two squares, the reference's square and the ratio add 5 u
+    from decimal import Decimal, getcontext
+    from paper_1505_07674_gb300 import lensed as LZ
+    from workloads import component, fixed, free
+    getcontext().prec = 40
+    comps = [component("gauss", "source", [fixed(0.0), fixed(0.0), fixed(0.8), free(0), fixed(0.7), fixed(0.0)])]
+    spec = {"nx": 1, "ny": 1, "h": 1.0, "rule": ("point", 1), "psf": None, "mask": None, "zeropoint": 0.0,
+            "components": comps, "n_params": 1}
+    mag = np.concatenate([[0.0], np.arange(-25.0, 26.0), np.random.default_rng(4).uniform(-25, 25, 1500)])
+    m = LZ.Model(spec, {"data": np.zeros((1, 1)), "variance": np.ones((1, 1))}, precision="fp64")
+    ll = m.loglike_batch(mag[:, None]).cpu().numpy()[0]
+    m.close()
+    u = 2.0 ** -53
+    for v, got in zip(mag, ll / ll[0]):
+        want = Decimal(10) ** (Decimal(-8) / Decimal(10) * Decimal(float(v)))
+        err = abs(float(Decimal(float(got)) / want - 1))
+        assert err <= u * (2 * (1.5 * np.log(10.0) * 0.4 * abs(v) + 5) + 5), (v, err / u)
