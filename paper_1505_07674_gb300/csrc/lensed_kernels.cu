@@ -1221,14 +1221,14 @@ __device__ __forceinline__ float pixel_rays(const KC &kc, const SysDev &S, int n
 template <int MODE, bool GQ>
 constexpr bool kTracePairs = MODE != LENSED_PREC_MIXED_FF || GQ;
 // Resident CTAs of 128 threads that the two-pixel kernels are compiled for: 6
-// (80 registers), and 5 (96) for the rows that spilled most at 80: 7 nodes
-// (chunks of 4 and 3 rays, both in the code) and guarded rows.  FP32,
-// two lenses, us a call, 6 / 5: one point of 64 x 64 pixels, 16 x 16 rays 175 /
-// 152, 11 x 11 103 / 91, 7 x 7 58 / 56; 22 points of 160 x 160, 16 x 16 rays 1,031 /
-// 1,024; 119 points, 7 x 7, work-queued 1,092 / 1,051.  Rows of 4 (a few bytes
-// spilled) are 2 % slower at 5.
+// (80 registers), and 5 (96) for guarded rows, which spill most at 80 (80 bytes
+// stored and loaded).  FP32, two lenses, us a call, 6 / 5: one point of 64 x 64
+// pixels, 16 x 16 rays 175 / 152, 11 x 11 103 / 91; 22 points of 160 x 160, 16 x 16
+// rays 1,031 / 1,024.  Rows of 4 and 7 spill up to 60 bytes at 80 registers and
+// are as fast or faster with them: 366 points of 160 x 160, 4 x 4 rays 1,064 /
+// 1,084; the 35-parameter lens with 7 x 7 rays, 256 points, 3,167 / 3,220.
 template <int G, bool EXACT>
-constexpr int kPairBlocks = EXACT && G != 7 ? 6 : 5;
+constexpr int kPairBlocks = EXACT ? 6 : 5;
 
 // trace_item for two pixels per thread: items start + t and start + t +
 // blockDim.x of the block.  Lanes without an item trace the block's last one

@@ -1,8 +1,9 @@
 """Register spills of the two-pixel trace kernels, all numbers of nodes per row, from
 the compiler (no GPU).
 
-A few bytes spilled outside the ray loop cost nothing that shows; the kernels that
-spilled more had lost to the one-pixel form in small launches.
+A few words spilled cost nothing that shows; the guarded rows, which spilled more, had
+lost to the one-pixel form in small launches.  Rows of 7 nodes are allowed twice as
+much: with the registers for it they were measured slower.
 """
 import os
 import re
@@ -45,4 +46,4 @@ TWO_PIXEL = ([f"Li0ELi{g}ELb1ELb0E" for g in range(1, 9)] + ["Li0ELi4ELb0ELb0E"]
 def test_two_pixel_kernels_spill_at_most_a_few_words(report, form, args):
     found = {k: v for k, v in report.items() if form + args in k}
     assert len(found) == 1, sorted(report)[:5]
-    assert max(found.values()) <= 32, found
+    assert max(found.values()) <= (64 if "Li7E" in args else 32), found
