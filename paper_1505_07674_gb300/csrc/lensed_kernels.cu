@@ -63,7 +63,8 @@ namespace lensed {
 // of a second pass are launched without it: their grids are sized to the whole
 // chip, and started as a trace drains, the first idle multiprocessors would
 // take most of their blocks (1,024 points of a 200 x 200 image, trace stage:
-// 1.65 ms so, 1.68 ms chained); so is the fix-up, but for the smallest launches.
+// 1.65 ms so, 1.68 ms chained); so are the fix-up and a trace that re-traces
+// rays in its blocks, but for small launches.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next()
 {
@@ -85,6 +86,14 @@ static void chain(void (*kernel)(K...), dim3 grid, unsigned threads, size_t smem
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
+
+// The same call for blocks that start when the kernel before has finished
+template <class... K, class... A>
+static void follow(void (*kernel)(K...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                   A &&...args)
+{
+    kernel<<<grid, threads, smem, st>>>(static_cast<K>(args)...);
 }
 
 // ---------------------------------------------------------------------------
@@ -1644,9 +1653,20 @@ static void trace_rows_t(int threads, const SysDev *sys, const int *comp_type,
     // (the work-queued form counts its items in 32 bits)
     if (!work || n_items > (1LL << 31)) {
         dim3 grid((unsigned)n_blocks, (unsigned)nP);
-        chain(k_trace_rows<MODE, G, EXACT, GQ>, grid, threads, 0, st, sys, comp_type,
-              comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0, (float *)Lbuf,
-              L_stride, fq);
+        // Blocks that re-trace their own rays (one pixel a thread) may take
+        // several times as long as others.  Placed while the prologue runs, they
+        // shared multiprocessors more unevenly than after it, which shows from
+        // two blocks per multiprocessor on (MIXED_FF, 24 x 24 pixels, us a call,
+        // chained / after it: 1,280 blocks, 16 x 16 rays, two lenses 1,681 / 1,509;
+        // 550 blocks, 8 x 8, one lens 209 / 187; 160 blocks, 9 x 9 191 / 206)
+        if (kTracePairs<MODE, GQ> || n_items <= 2 * g_sm_count)
+            chain(k_trace_rows<MODE, G, EXACT, GQ>, grid, threads, 0, st, sys, comp_type,
+                  comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0, (float *)Lbuf,
+                  L_stride, fq);
+        else
+            follow(k_trace_rows<MODE, G, EXACT, GQ>, grid, threads, 0, st, sys, comp_type,
+                   comp_plane, cf, cd, valid, P, C_total, blocks, need, nodes, p0, (float *)Lbuf,
+                   L_stride, fq);
         return;
     }
     int per_sm = 0;
@@ -2023,8 +2043,8 @@ void launch_fix64(LaunchCfg cfg, const SysDev *sys, int s0, int nS, const int *c
         chain(k_trace_fix64, grid, 128, 0, st, sys, s0, comp_type, comp_plane, cf, cd, valid, P,
               C_total, need, nodes, p0, (float *)Lbuf, L_stride);
     else
-        k_trace_fix64<<<grid, 128, 0, st>>>(sys, s0, comp_type, comp_plane, cf, cd, valid, P,
-                                            C_total, need, nodes, p0, (float *)Lbuf, L_stride);
+        follow(k_trace_fix64, grid, 128, 0, st, sys, s0, comp_type, comp_plane, cf, cd, valid, P,
+               C_total, need, nodes, p0, (float *)Lbuf, L_stride);
 }
 
 // ---------------------------------------------------------------------------
