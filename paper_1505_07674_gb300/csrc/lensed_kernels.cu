@@ -1053,19 +1053,6 @@ __device__ __forceinline__ float light_f32_rho(const LightF &k, float x, float y
 
 constexpr int kQCap = 2048;       // deferred float-float rays per trace block
 
-// a2-a5 in FP32 (also the first pass of MIXED): one thread per pixel; for
-// every row of the rule's node grid, G rays are traced together component by
-// component, so each component's constants are read into registers once per
-// G rays and the G independent rays give the scheduler instruction-level
-// parallelism.  EXACT: the rule has exactly G nodes per row (no guards).
-// GQ (MIXED_FF, EXACT): the float-float re-traces go to the launch's global
-// queue, appended warp by warp, for k_retrace_ff and k_apply_ff.
-// What a pixel's ray loop does with rays near the centre of a Sersic-type
-// source (MIXED_FF): nothing (other modes), record the smallest (R/r)^2 of
-// all rays in pmin, defer the rays' source light to the queue (their bits in
-// mask; the rest of the light summed now), or re-trace them in place.
-constexpr int kNearIgnore = 0, kNearFlag = 1, kNearDefer = 2, kNearInPlace = 3;
-
 // Where a pixel's ray loop reads its point's constants: the trace block's
 // staged copy in shared memory, or global memory (a pixel of any point).
 struct SmemConsts {
@@ -1101,10 +1088,14 @@ struct GlobalConsts {
 // component (each component's constants read once per G rays), two at a
 // time in packed FP32 instructions, each ray's brightness added to acc with
 // its weight in ray order.  EXACT: the rule has exactly G nodes per row.
-template <int MODE, int G, bool EXACT, int NEAR, class KC>
+// MIXED_FF only (the other modes trace two pixels per thread,
+// lensed_pair.cuh): the source light of rays near the centre of a Sersic-type
+// source is left to a queue (DEFER: their bits in mask, the rest of the light
+// summed now) or re-traced in place.
+template <int G, bool EXACT, bool DEFER, class KC>
 __device__ __forceinline__ float pixel_rays(const KC &kc, const SysDev &S, int ncomp, int nn,
                                             float jc, float ic, float acc,
-                                            unsigned long long &mask, float &pmin)
+                                            unsigned long long &mask)
 {
     // pixel centre (j - cx) h with h as a float pair: one rounding, no
     // coherent scale error
@@ -1182,13 +1173,12 @@ __device__ __forceinline__ float pixel_rays(const KC &kc, const SysDev &S, int n
                         using V = std::remove_reference_t<decltype(i)>;
                         i = vadd(i, vsplat<V>(L.A));
                     }, I);
-                } else if (NEAR != kNearIgnore && L.kind == (float)kKindPower) {
+                } else if (L.kind == (float)kKindPower) {
                     for_rays<G>([&](auto &x, auto &dx, auto &dy, auto &i, auto &rm) {
                         using V = std::remove_reference_t<decltype(x)>;
                         V r2;
                         i = vadd(i, light_at_v(L, vsub(x, dx), vsub(vsplat<V>(y), dy), &r2));
-                        if (NEAR == kNearFlag) pmin = fminf(pmin, vminlane(r2));
-                        else rm = vmap(rm, r2, [](float p, float q) { return fminf(p, q); });
+                        rm = vmap(rm, r2, [](float p, float q) { return fminf(p, q); });
                     }, xk, ax, ay, I, rmin);
                 } else {
                     for_rays<G>([&](auto &x, auto &dx, auto &dy, auto &i) {
@@ -1197,7 +1187,7 @@ __device__ __forceinline__ float pixel_rays(const KC &kc, const SysDev &S, int n
                     }, xk, ax, ay, I);
                 }
             }
-            if (NEAR == kNearDefer) {
+            if (DEFER) {
                 // the source part comes from the queue; keep the rest (the
                 // row's flags gathered first, one shift into the mask per row)
                 unsigned row = 0u;
@@ -1208,7 +1198,7 @@ __device__ __forceinline__ float pixel_rays(const KC &kc, const SysDev &S, int n
                     I.set(k, nk ? Ifg.get(k) : I.get(k));
                 }
                 mask |= (unsigned long long)row << (b * nn);
-            } else if (NEAR == kNearInPlace) {
+            } else {
 #pragma unroll
                 for (int k = 0; k < G; ++k) {
                     if (!(rmin.get(k) < kCuspRho2) || !(EXACT || a0 + k < nn)) continue;
@@ -1241,7 +1231,7 @@ constexpr int kPairBlocks = EXACT ? 6 : 5;
 
 // trace_item for two pixels per thread: items start + t and start + t +
 // blockDim.x of the block.  Lanes without an item trace the block's last one
-// and write nothing (the warp votes on the form of atanh, so all lanes run).
+// and write nothing.
 template <int G, bool EXACT, bool GQ>
 __device__ __forceinline__ void pair_item(PairSmem &sm, const SysDev *__restrict__ sys,
                                           const int *__restrict__ comp_type,
@@ -1303,7 +1293,8 @@ __device__ __forceinline__ void pair_item(PairSmem &sm, const SysDev *__restrict
 // The work of one trace block tb at point p (every thread of the CTA calls
 // it; it returns to the caller, which may take another item).  stage = false:
 // the shared constants already hold tb's system at point p.
-template <int MODE, int G, bool EXACT>
+// MIXED_FF with its re-traces in the block: one pixel per thread.
+template <int G, bool EXACT>
 __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
                                            const int *__restrict__ comp_type,
                                            const int *__restrict__ comp_plane,
@@ -1320,10 +1311,10 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
     if (!valid[(size_t)tb.sys * P + p]) return;
     const SysDev &S = sys[tb.sys];
     const size_t cbase = ((size_t)p * C_total + S.comp_off) * kNC;
-    // MIXED_FF with at most 8 nodes per row defers its float-float re-traces
-    // (64-bit ray mask per pixel) to a block-wide queue processed by all
-    // lanes after the main loop; with more it re-traces in place
-    constexpr bool kQueue = (MODE == LENSED_PREC_MIXED_FF) && EXACT;
+    // at most 8 nodes per row: the float-float re-traces are deferred (64-bit
+    // ray mask per pixel) to a block-wide queue processed by all lanes after
+    // the main loop; with more they run in place
+    constexpr bool kQueue = EXACT;
     __shared__ int q_n;
     __shared__ unsigned short q_t[kQueue ? kQCap : 1];
     __shared__ unsigned char q_r[kQueue ? kQCap : 1];
@@ -1344,13 +1335,8 @@ __device__ __forceinline__ void trace_item(const SysDev *__restrict__ sys,
 
     float acc = (nodes.pre_f && S.pre_off >= 0 && active) ? nodes.pre_f[S.pre_off + pix] : 0.f;
     unsigned long long mask = 0ull;  // rays deferred to the queue
-    float pmin = kCuspRho2;          // smallest (R/r)^2 of the pixel's rays
-    constexpr int kNear = MODE != LENSED_PREC_MIXED_FF ? kNearIgnore
-                        : !EXACT                     ? kNearInPlace
-                                                     : kNearDefer;
     if (active)
-        acc = pixel_rays<MODE, G, EXACT, kNear>(SmemConsts{sm}, S, ncomp, nn, jc, ic, acc, mask,
-                                                pmin);
+        acc = pixel_rays<G, EXACT, kQueue>(SmemConsts{sm}, S, ncomp, nn, jc, ic, acc, mask);
     if (kQueue) {
         // each pixel's deferred rays take consecutive slots in ray order
         const int n_t = __popcll(mask);
@@ -1407,7 +1393,7 @@ __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs
                                 p0, Lbuf, L_stride, fq, blocks[blockIdx.x], p0 + (int)blockIdx.y,
                                 true);
     } else {
-        trace_item<MODE, G, EXACT>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total, need,
+        trace_item<G, EXACT>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total, need,
                                    nodes, p0, Lbuf, L_stride, blocks[blockIdx.x],
                                    p0 + (int)blockIdx.y);
     }
@@ -1457,7 +1443,7 @@ __global__ void __launch_bounds__(kTracePairs<MODE, GQ> ? 128 : 256, kTracePairs
                 pair_item<G, EXACT, GQ>(sm, sys, comp_type, comp_plane, cf, valid, P, C_total, need,
                                         nodes, p0, Lbuf, L_stride, fq, tb, p0 + (int)q, stage);
             else
-                trace_item<MODE, G, EXACT>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total,
+                trace_item<G, EXACT>(sys, comp_type, comp_plane, cf, cd, valid, P, C_total,
                                            need, nodes, p0, Lbuf, L_stride, tb, p0 + (int)q, stage);
             __syncthreads();  // the item is done with the shared arrays
         }
@@ -1506,11 +1492,10 @@ __global__ void __launch_bounds__(kFfThreads)
                              nodes.u + S.node_off, nodes.ul + S.node_off,
                              nodes.w + S.w2_off};
         unsigned long long mask = 0ull;
-        float acc = 0.f, pmin = kCuspRho2;
+        float acc = 0.f;
         if (active) {
             acc = (nodes.pre_f && S.pre_off >= 0) ? nodes.pre_f[S.pre_off + pix] : 0.f;
-            acc = pixel_rays<LENSED_PREC_MIXED_FF, G, true, kNearDefer>(K, S, S.ncomp, G, jc, ic,
-                                                                       acc, mask, pmin);
+            acc = pixel_rays<G, true, true>(K, S, S.ncomp, G, jc, ic, acc, mask);
         }
         const int n_t = __popcll(mask);
         if (__any_sync(full, n_t != 0)) {

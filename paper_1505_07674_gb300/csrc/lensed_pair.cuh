@@ -40,7 +40,6 @@ constexpr float kCuspRho2 = 0.25f;
 constexpr int kPairNC = 28;
 constexpr int kPairNSn = 24, kPairNSnL = 25;
 
-constexpr int kPairThreads = 128;  // most threads of a CTA
 constexpr int kPairW = 8;  // row stride of the staged 2-D weights (16-byte rows)
 
 struct PairSmem {

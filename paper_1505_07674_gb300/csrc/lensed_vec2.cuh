@@ -69,10 +69,6 @@ __device__ __forceinline__ float2 vmap(float2 a, float2 b, float2 c, float2 d, F
     return make_float2(f(a.x, b.x, c.x, d.x), f(a.y, b.y, c.y, d.y));
 }
 
-// smallest lane
-__device__ __forceinline__ float vminlane(float a) { return a; }
-__device__ __forceinline__ float vminlane(float2 a) { return fminf(a.x, a.y); }
-
 // G rays' values: G / 2 pairs and, for odd G, one single ray (the last)
 template <int G>
 struct Rays {
