@@ -343,7 +343,9 @@ int lensed_eval_sie_trig(const float *n, const float *d, long long count, float 
  * persistent, work-queued launch.  LENSED_PREC_MIXED_FF: n = 24, and
  * 12 + k runs configuration k with the float-float re-traces in a second
  * pass.  The default is 0; for LENSED_PREC_MIXED_FF 12, with the re-traces
- * inside the trace blocks in launches too small for a second pass to pay. */
+ * inside the trace blocks in launches too small for a second pass to pay.
+ * (0 takes up to a quarter less time where sources fill much of a small image;
+ * lensed_autotune finds out.) */
 int lensed_set_config(lensed_model *m, int index);
 
 /* Points per scratch chunk of the batched schedule (a8; the paper has no

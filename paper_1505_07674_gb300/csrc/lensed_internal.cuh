@@ -124,7 +124,15 @@ struct LaunchCfg {
 // launches.  A call in ms, in-block / second pass, by blocks of the launch:
 // 64 x 64, 5 x 5 rays: 4,096 .162/.170, 8,192 .262/.252; 200 x 200: 10,016
 // .146/.155, 20,032 .224/.220; 400 x 400: 10,000 .252/.266, 20,000 .454/.440;
-// 160 x 160, 7 x 7 rays, two lenses: 3,200 .326/.334, 6,400 .540/.531.
+// 160 x 160, 7 x 7 rays, two lenses: 3,200 .326/.334, 6,400 .540/.531.  The two
+// meet anywhere between 3,200 and 20,000 blocks, by rays and components; the
+// line lies where neither loses more than 6 %.
+// How many rays a source's centre takes matters more, and no call knows it
+// beforehand.  Second pass / in-block, 25,600 blocks of one lens and one source
+// of effective radius .2, .4, .7, 1, 3 arcsec: 64 x 64 pixels of 0.05 arcsec,
+// 5 x 5 rays .85, 1.03, 1.13, .89, 1.07, 3 x 3 .79, .93, 1.08, 1.15, 1.37, 7 x 7
+// .84, .79, .67, .84, 1.09; 160 x 160, 5 x 5 .85, .88, .93, .98, 1.01.  Sources
+// that fill a small image want configuration 0, or the autotuner.
 constexpr long long kSecondPassBlocks = 10240;
 inline bool second_pass(LaunchCfg cfg, int nn, long long blocks)
 {

@@ -56,15 +56,15 @@ namespace lensed {
 // blocks have started and called chain_next, or exited), so its launch and
 // prologue cost no gap.  Every block calls chain_wait before it touches
 // anything that an earlier kernel of the stream, the one before or any other,
-// reads or writes: that returns
-// when the earlier kernel has completed, which by the same rule has waited for
-// the one before it.  Eight points of a 64 x 64 image, a call: 87 us launch by
-// launch, 69 us so; a render with its error map: 283 and 212 us.  The kernels
-// of a second pass are launched without it: their grids are sized to the whole
-// chip, and started as a trace drains, the first idle multiprocessors would
-// take most of their blocks (1,024 points of a 200 x 200 image, trace stage:
-// 1.65 ms so, 1.68 ms chained); so are the fix-up and a trace that re-traces
-// rays in its blocks, but for small launches.
+// reads or writes: that returns when the earlier kernel has completed, which by
+// the same rule has waited for the one before it.  A render with its error map:
+// 281 us launch by launch, 257 us so; eight points of a 64 x 64 image through
+// host buffers: 91 and 90 us.  The kernels of a second pass are launched
+// without it: their grids are sized to the whole chip, and started as a trace
+// drains, the first idle multiprocessors would take most of their blocks (1,024
+// points of a 200 x 200 image, trace stage: 1.65 ms so, 1.68 ms chained); so are
+// the fix-up and a trace that re-traces rays in its blocks, but for small
+// launches.
 __device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void chain_next()
 {

@@ -15,10 +15,12 @@
 //     5 packed operations more than branching, but no branch splits the C
 //     chains, which lets them overlap in 80 registers (6 warps per
 //     scheduler).
-// Measured on the 200x200 workload (5 x 5 rule, 512 points): 79.9 warp
-// instructions per ray instead of 124.5 with rays paired inside a row, first
-// pass 676 instead of 888 us; the FMA pipe is 72 % busy (45 packed operations
-// of two cycles each per ray), the issue slots 64 %.
+// Measured on the 200x200 workload (5 x 5 rule, 512 points): 87 warp
+// instructions per 32 rays, 44 of them packed, first pass 705 us; 941 us with
+// one pixel per thread.  A packed operation takes two issue slots: 131 of the
+// 131 scheduler cycles per 32 rays.  7 x 7 rays, eight components: 91 % of the
+// cycles; the rest waits for instructions (0.81 such stalls per issue, 0.17
+// with the 5 x 5 rule): its code holds a chunk of 4 and one of 3 rays.
 #pragma once
 
 #include "lensed_internal.cuh"
